@@ -474,6 +474,16 @@ void record(hsma_plan_s *p, cudaStream_t st, int i)
     if (p->profile && p->events_ready) cudaEventRecord(p->ev[i], st);
 }
 
+// Fixed-point ranges of the FP64 near sums: the in-set lies inside Rs,
+// particles inside the box (reused in-sets: and the skin), monitoring points
+// inside the circumsphere.
+void pair_ranges(const hsma_plan_s *p, PairArgs &pa)
+{
+    const double half = 0.5 * std::max(p->L[0], std::max(p->L[1], p->L[2]));
+    pa.fx_part = pair_fx_range(p->Rs, half + p->md_skin);
+    pa.fx_ext = pair_fx_range(p->Rs, p->bc == HSMA_BC_PERIODIC ? p->R0 * 1.000001 : half);
+}
+
 // Every kernel of the update step, enqueued on `st`.  Reads its inputs from
 // the workspace staging buffers and writes forces/potentials to the staging
 // outputs, so the same sequence can be captured once into a CUDA graph and
@@ -600,6 +610,7 @@ int enqueue_update(hsma_plan_s *p, const BatchShape &sh, const Workspace &w, int
     pa.ext_boxes = w.boxes ? (TB == 256 ? p->mon_boxes2 : (TB == 384 ? p->mon_boxes3 : p->mon_boxes)) : nullptr;
     pa.stall_test = p->stall_test;
     pa.far2 = (float)(p->far_rel * p->Rs * p->far_rel * p->Rs);
+    pair_ranges(p, pa);
     pa.partials = w.partials;
     pa.next_item = w.ctrl;
     pa.status = w.status;
@@ -1044,6 +1055,7 @@ int run_shard(hsma_plan_s *p, const hsma_particles *x, bool far_stage, int part,
         pa.boxes = w.boxes;
         pa.ext_boxes = w.boxes ? (TB == 256 ? p->mon_boxes2 : (TB == 384 ? p->mon_boxes3 : p->mon_boxes)) : nullptr;
         pa.far2 = (float)(p->far_rel * p->Rs * p->far_rel * p->Rs);
+        pair_ranges(p, pa);
         pa.partials = w.partials;
         pa.next_item = w.ctrl;
         pa.status = w.status;

@@ -397,6 +397,14 @@ struct RegenArgs {
 int launch_inset_regen(const RegenArgs &r, cudaStream_t st);
 
 // pair.cu
+// Fixed-point formats of the FP64 sums (pair_fx.cuh).  scale: a power of two,
+// coordinates times scale 2^30 are the integers h, sources within +-src_lim
+// (targets within 2^31 - 1 - src_lim); scale 0: native FP64 throughout.
+struct FxRange {
+    double scale = 0.0;
+    double src_lim = 0.0;
+};
+
 struct PairArgs {
     const SysDesc *sys;
     int nsys;
@@ -417,6 +425,7 @@ struct PairArgs {
     float far2 = 0.f;               // tiles at least sqrt(far2) from the target block skip the low words
     int one_item = 0;               // 1: CTA b does work item b and exits (grid = total_items), so that
                                     // work on other streams gets SMs between items
+    FxRange fx_part, fx_ext;  // FP64 form: formats for particle and for external targets
     float4 *partials;       // 2 x float4 (FP32) or 1 x double4_32a (FP64) per record
     int *next_item;
     int *status;
@@ -424,6 +433,9 @@ struct PairArgs {
 // variant (FP32 form): one of the codes pair_variant_valid accepts; it fixes
 // the targets per thread -- 4 (blocks and tiles of 512), 3 (384) or 2 (256) --
 // the inner loop (scalar or packed f32x2) and the CTAs per SM.
+// The formats for source coordinates of magnitude up to r_src and target
+// coordinates up to r_tgt.
+FxRange pair_fx_range(double r_src, double r_tgt);
 int launch_pair(const PairArgs &a, int precision, int variant, int grid, cudaStream_t st);
 bool pair_variant_valid(int variant);
 int pair_targets_per_block(int precision, int variant = 4);

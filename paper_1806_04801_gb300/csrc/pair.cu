@@ -22,8 +22,14 @@
 // variants run the same arithmetic on two sources per f32x2 instruction
 // (fma/add/mul.rn.f32x2), which halves the issue slots of the FP32 work.
 //
-// FP64 form: the same loop in double, rsqrt() from the CUDA math library.
+// FP64 form: the same decomposition; the pairs are summed in fixed point on
+// the integer and FP32 pipes (pair_fx.cuh), close pairs in native FP64.
+#include <algorithm>
+#include <cmath>
+#include <cstdlib>
+
 #include "common.cuh"
+#include "pair_fx.cuh"
 
 namespace hsma {
 
@@ -36,6 +42,7 @@ constexpr int kThreads = 128;
 constexpr int kT64 = 2;
 constexpr int kTB64 = kThreads * kT64;
 constexpr int kTile64 = 256;
+constexpr int kFoldFx = 16;             // FxSums::gf fold interval (sources)
 constexpr int kFold = 32;               // potential fold interval (sources)
 constexpr int kFold2 = 64;              // packed loop: 32 sources per lane
 constexpr bool kCpDouble = true;        // mode 1: two interleaved buffers, one barrier per tile
@@ -506,40 +513,172 @@ __global__ void __launch_bounds__(kThreads, MINB) pair_fp32_kernel(PairArgs a)
 }
 
 // ------------------------------------------------------------ FP64 tiles
-template <bool FIELD, int SKIP>
-__device__ __forceinline__ void tile64(const double4_32a *__restrict__ s4, int cnt, const double (&tx)[kT64][3],
-                                       const int (&self_rel)[kT64], double (&phi)[kT64], double (&g)[kT64][3])
+// The FP64 sums run on the integer and FP32 pipes (pair_fx.cuh has the
+// arithmetic and the reason); pairs outside its formats take native FP64.
+// A CTA turns each staged tile into fixed point once (36 FP64 operations per
+// source for 256 targets) with the charges scaled by the tile's largest, and
+// sums it for two targets per thread; the tile's integer sums go to FP64
+// accumulators in shared memory.  Near pairs are a few in a thousand, but
+// some lane has one in 1-3% of a warp's steps; they use the otherwise idle
+// FP64 pipe while other warps go on (14% busy), so a larger near radius would
+// cost little and a smaller one would cost the field's precision.
+// Bound by the FMA-heavy pipe, which issues the 32 x 32 multiplies (78% of
+// its active cycles; ALU 44%, issue slots 64%).  Measured: near-sum phase of
+// N = 9999 (1.96e9 pairs) 61.3 -> 11.0 ms, 3.2e10 -> 1.78e11 pairs/s; N = 1000
+// 1.30 -> 0.32 ms; grounded N = 3001 9.4 -> 1.8 ms.  Error against quad
+// precision (N = 300..4000, both boundaries, three charge patterns): field
+// 1.9e-16..8.2e-16 of its norm against 4.7e-16..1.7e-15 before, potential
+// 1.3e-16..3.9e-15 against 3.5e-16..5.2e-15.
+struct FxShared {
+    double4_32a src[2][kTile64];       // staged sources (bulk copies land here)
+    FxSource fx[kTile64];              // the tile being summed, in fixed point
+    double tgt[kT64][3][kThreads];     // this block's targets
+    double acc[kT64][4][kThreads];     // their potential and field sums
+    float2 gf[kT64][3][kThreads];      // double-float sums of FxSums::gf of a tile
+    unsigned qmax[2][kThreads / 32], qmin[2][kThreads / 32];
+};
+
+// |v| as the upper word of its bits (ordered like |v|).
+__device__ __forceinline__ unsigned abs_hi(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+
+// 2^k, -1022 <= k <= 1023.
+__device__ __forceinline__ double exp2i(int k) { return __hiloint2double((k + 1023) << 20, 0); }
+
+// One pair in native FP64, added to this thread's sums.  skip: the target's
+// own slot; skip_zero: leave out a pair at distance exactly zero.
+template <bool FIELD>
+__device__ __forceinline__ void pair64(const double4_32a &p, double tx, double ty, double tz, bool skip,
+                                       bool skip_zero, double &phi, double &gx, double &gy, double &gz)
 {
+    const double dx = p.x - tx, dy = p.y - ty, dz = p.z - tz;
+    const double r2 = dx * dx + dy * dy + dz * dz;
+    double ri = rsqrt(r2);
+    if (skip || (skip_zero && !(r2 > 0.0))) ri = 0.0;
+    const double qr = p.w * ri;
+    phi += qr;
+    if (FIELD) {
+        const double qr3 = qr * ri * ri;
+        gx += qr3 * dx;
+        gy += qr3 * dy;
+        gz += qr3 * dz;
+    }
+}
+
+// A tile in native FP64: charges or coordinates outside the fixed-point
+// formats, or (mostly) near pairs.
+template <bool FIELD>
+__device__ __noinline__ void tile64(FxShared &sm, int buf, int cnt, const int (&self_rel)[kT64], bool skip_zero)
+{
+    const int tid = threadIdx.x;
+    double tx[kT64][3], g[kT64][4];
+#pragma unroll
+    for (int t = 0; t < kT64; ++t) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) tx[t][c] = sm.tgt[t][c][tid];
+        g[t][0] = g[t][1] = g[t][2] = g[t][3] = 0.0;
+    }
 #pragma unroll 2
     for (int s = 0; s < cnt; ++s) {
-        const double4_32a p = s4[s];
+        const double4_32a p = sm.src[buf][s];
+#pragma unroll
+        for (int t = 0; t < kT64; ++t)
+            pair64<FIELD>(p, tx[t][0], tx[t][1], tx[t][2], s == self_rel[t], skip_zero, g[t][0], g[t][1], g[t][2],
+                          g[t][3]);
+    }
+#pragma unroll
+    for (int t = 0; t < kT64; ++t)
+#pragma unroll
+        for (int c = 0; c < (FIELD ? 4 : 1); ++c) sm.acc[t][c][tid] += g[t][c];
+}
+
+// A tile in fixed point.  ps, gs: factors of the potential and field sums.
+// Returns how many of the cnt source steps held a near pair in this warp.
+template <bool FIELD>
+__device__ __forceinline__ int tile_fx(FxShared &sm, int buf, int cnt, const FxTarget (&tg)[kT64],
+                                       const int (&self_rel)[kT64], bool skip_zero, double ps, double gs)
+{
+    const int tid = threadIdx.x;
+    FxSums sums[kT64];
+#pragma unroll
+    for (int t = 0; t < kT64; ++t) {
+        fx_clear(sums[t]);
+        if (FIELD) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) sm.gf[t][c][tid] = make_float2(0.f, 0.f);
+        }
+    }
+    int slow = 0;
+    auto fold = [&]() {
+#pragma unroll
+        for (int t = 0; t < kT64; ++t)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                sm.gf[t][c][tid] = df_add(sm.gf[t][c][tid], sums[t].gf[c]);
+                sums[t].gf[c] = 0.f;
+            }
+    };
+#pragma unroll 1
+    for (int s = 0; s < cnt; ++s) {
+        // one FP32 sum over the whole tile would round every term at the
+        // closest pairs' magnitude
+        if (FIELD && s % kFoldFx == 0) fold();
+        const FxSource f = sm.fx[s];
+        const int qsign = f.qh >> 31;
+        int dh[kT64][3];
+        uint64_t A[kT64];
+        bool any = false;
 #pragma unroll
         for (int t = 0; t < kT64; ++t) {
-            double dx = p.x - tx[t][0];
-            double dy = p.y - tx[t][1];
-            double dz = p.z - tx[t][2];
-            double r2 = dx * dx + dy * dy + dz * dz;
-            double ri = rsqrt(r2);
-            if (SKIP == 1) ri = (s == self_rel[t]) ? 0.0 : ri;
-            if (SKIP == 2) ri = (r2 > 0.0) ? ri : 0.0;
-            double qr = p.w * ri;
-            phi[t] += qr;
+            dh[t][0] = f.hx - tg[t].h[0];
+            dh[t][1] = f.hy - tg[t].h[1];
+            dh[t][2] = f.hz - tg[t].h[2];
+            const int dl[3] = {f.lx - tg[t].l[0], f.ly - tg[t].l[1], f.lz - tg[t].l[2]};
+            A[t] = fx_distance2(dh[t], dl);
+            any = any || A[t] < kFxNearA;
+        }
+        if (any) {
+            ++slow;
+            const double4_32a p = sm.src[buf][s];
+#pragma unroll
+            for (int t = 0; t < kT64; ++t) {
+                if (A[t] < kFxNearA)
+                    pair64<FIELD>(p, sm.tgt[t][0][tid], sm.tgt[t][1][tid], sm.tgt[t][2][tid], s == self_rel[t],
+                                  skip_zero, sm.acc[t][0][tid], sm.acc[t][1][tid], sm.acc[t][2][tid],
+                                  sm.acc[t][3][tid]);
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < kT64; ++t) {
+            const FxPair r = fx_inverse(A[t], A[t] < kFxNearA, f.qh, f.ql);
+            fx_add_potential(sums[t], r, f.fq);
             if (FIELD) {
-                double qr3 = qr * ri * ri;
-                g[t][0] += qr3 * dx;
-                g[t][1] += qr3 * dy;
-                g[t][2] += qr3 * dz;
+                const float df[3] = {f.fx - tg[t].f[0], f.fy - tg[t].f[1], f.fz - tg[t].f[2]};
+                fx_add_field(sums[t], r, dh[t], df, qsign, f.fq);
             }
         }
     }
+    if (FIELD) fold();
+#pragma unroll
+    for (int t = 0; t < kT64; ++t) {
+        sm.acc[t][0][tid] += fx_potential(sums[t]) * ps;
+        if (FIELD) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float2 g = sm.gf[t][c][tid];
+                sm.acc[t][1 + c][tid] += fx_field(sums[t], c, (double)g.x + (double)g.y) * gs;
+            }
+        }
+    }
+    return __reduce_max_sync(0xffffffffu, slow);
 }
 
 __global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
 {
-    extern __shared__ __align__(128) double4_32a smem64[];  // [2][kTile64]
+    extern __shared__ __align__(128) unsigned char smem64[];
+    FxShared &sm = *reinterpret_cast<FxShared *>(smem64);
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ int s_item, s_abort;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
     if (tid == 0) {
         mbar_init(&bar[0], 1);
         mbar_init(&bar[1], 1);
@@ -548,7 +687,6 @@ __global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
     }
     __syncthreads();
     uint32_t parity[2] = {0u, 0u};
-
     for (int round = 0;; ++round) {
         if (tid == 0) s_item = a.one_item ? (round == 0 ? (int)blockIdx.x : a.total_items) : atomicAdd(a.next_item, 1);
         __syncthreads();
@@ -562,28 +700,14 @@ __global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
         const int t1 = (int)((it.chunk + 1) * ntiles / sd.nchunks);
         const bool part = it.tb < sd.ntb_part;
         const bool field = part || a.ext_field;
+        const bool skip_zero = !part && a.ext_skip_zero;
         const long long ntgt = sd.n + a.n_ext;
         const int gb = part ? sd.pb_lo + it.tb : sd.mb_lo + it.tb - sd.ntb_part;
 
-        double tx[kT64][3];
-        long long tidx[kT64];
-        long long tb_lo = 0, tb_hi = 0;
-        if (part) {
-            tb_lo = (long long)gb * kTB64;
-            tb_hi = tb_lo + kTB64;
-        }
-#pragma unroll
-        for (int t = 0; t < kT64; ++t) {
-            long long k = (long long)gb * kTB64 + t * kThreads + tid;
-            bool valid = part ? (k < sd.n) : (k < a.n_ext);
-            double4_32a p = make_double4_32a(1e4, 1e4, 1e4, 0.0);
-            if (valid) p = part ? a.src64[sd.src_off + k] : a.ext64[k];
-            tx[t][0] = p.x; tx[t][1] = p.y; tx[t][2] = p.z;
-            tidx[t] = valid ? (part ? k : sd.n + k) : -1;
-        }
-        double phi[kT64], g[kT64][3];
-#pragma unroll
-        for (int t = 0; t < kT64; ++t) phi[t] = g[t][0] = g[t][1] = g[t][2] = 0.0;
+        // fixed-point formats of this item: coordinates times `unit`, sources
+        // within +-src_lim, targets within +-tgt_lim
+        const FxRange rg = part ? a.fx_part : a.fx_ext;
+        const double unit = rg.scale * 0x1p30, src_lim = rg.src_lim, tgt_lim = 2147483647.0 - src_lim;
 
         const double4_32a *gs = a.src64 + sd.src_off;
         const int ntile = t1 - t0;
@@ -593,12 +717,38 @@ __global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
             uint32_t bytes = (uint32_t)cnt * 32u;
             fence_proxy_async_smem();
             mbar_arrive_expect_tx(&bar[buf], bytes);
-            bulk_g2s(smem64 + buf * kTile64, gs + s0, bytes, &bar[buf]);
+            bulk_g2s(sm.src[buf], gs + s0, bytes, &bar[buf]);
         };
         if (tid == 0) {
             if (ntile > 0) issue(0, 0);
             if (ntile > 1) issue(1, 1);
         }
+        FxTarget tg[kT64];
+        long long tidx[kT64];
+        bool outside = false;
+#pragma unroll
+        for (int t = 0; t < kT64; ++t) {
+            long long k = (long long)gb * kTB64 + t * kThreads + tid;
+            bool valid = part ? (k < sd.n) : (k < a.n_ext);
+            // slots past the last target repeat it, unwritten
+            if (!valid) k = (part ? sd.n : (long long)a.n_ext) - 1;
+            const double4_32a p = part ? gs[k] : a.ext64[k];
+            sm.tgt[t][0][tid] = p.x;
+            sm.tgt[t][1][tid] = p.y;
+            sm.tgt[t][2][tid] = p.z;
+            const double v[3] = {p.x * unit, p.y * unit, p.z * unit};
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                outside |= !(fabs(v[c]) <= tgt_lim + 1.0);
+                fx_split(v[c], tgt_lim, tg[t].h[c], tg[t].l[c], tg[t].f[c]);
+            }
+            tidx[t] = valid ? (part ? k : sd.n + k) : -1;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) sm.acc[t][c][tid] = 0.0;
+        }
+        const bool blk_native = __syncthreads_or(outside || !(unit > 0.0));
+        int native_tiles = 0;  // this warp's next tiles go native: the last one held mostly near pairs
+
         for (int k = 0; k < ntile; ++k) {
             const int buf = k & 1;
             if (!mbar_wait_bounded(&bar[buf], parity[buf])) {
@@ -606,27 +756,67 @@ __global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
                 atomicOr(&a.status[it.sys], ST_TIMEOUT);
             }
             parity[buf] ^= 1u;
-            __syncthreads();
-            if (s_abort) break;
             const long long s0 = (long long)(t0 + k) * kTile64;
             const int cnt = (int)min((long long)kTile64, Ns - s0);
-            const double4_32a *b4 = smem64 + buf * kTile64;
-            const int skip = part ? ((s0 < tb_hi && s0 + cnt > tb_lo) ? 1 : 0) : (a.ext_skip_zero ? 2 : 0);
             int self_rel[kT64];
 #pragma unroll
-            for (int t = 0; t < kT64; ++t) self_rel[t] = (int)(tidx[t] - s0);
-            if (field) {
-                if (skip == 1)
-                    tile64<true, 1>(b4, cnt, tx, self_rel, phi, g);
-                else if (skip == 2)
-                    tile64<true, 2>(b4, cnt, tx, self_rel, phi, g);
+            for (int t = 0; t < kT64; ++t) {
+                const long long o = part && tidx[t] >= 0 ? tidx[t] - s0 : -1;
+                self_rel[t] = o >= 0 && o < kTile64 ? (int)o : -1;
+            }
+            // charge range of the tile; 0x7fffffff marks what the formats do not hold
+            unsigned qmax = 0u, qmin = 0x7fffffffu;
+            for (int s = tid; s < cnt; s += kThreads) {
+                const double4_32a p = sm.src[buf][s];
+                const unsigned hq = abs_hi(p.w);
+                const bool ok = fabs(p.x * unit) <= src_lim + 1.0 && fabs(p.y * unit) <= src_lim + 1.0 &&
+                                fabs(p.z * unit) <= src_lim + 1.0 && hq < 0x7ff00000u &&
+                                (hq >= 0x00100000u || p.w == 0.0);
+                qmax = max(qmax, ok ? hq : 0x7fffffffu);
+                if (p.w != 0.0) qmin = min(qmin, hq);
+            }
+            qmax = __reduce_max_sync(0xffffffffu, qmax);
+            qmin = __reduce_min_sync(0xffffffffu, qmin);
+            if (lane == 0) {
+                sm.qmax[buf][wid] = qmax;
+                sm.qmin[buf][wid] = qmin;
+            }
+            __syncthreads();
+            if (s_abort) break;
+#pragma unroll
+            for (int w = 0; w < kThreads / 32; ++w) {
+                qmax = max(qmax, sm.qmax[buf][w]);
+                qmin = min(qmin, sm.qmin[buf][w]);
+            }
+            // the largest |q| scaled to [1/2, 1); the smallest must keep its
+            // bits next to it (a target that skips the largest sees only the others)
+            int eq = qmax == 0u ? 1022 : (int)(qmax >> 20);
+            const bool native =
+                blk_native || eq > 1923 || eq < 123 || (qmax != 0u && (int)(qmin >> 20) < eq - 20);
+            if (!native) {
+                const double qs = exp2i(1022 - eq);
+                for (int s = tid; s < cnt; s += kThreads) {
+                    const double4_32a p = sm.src[buf][s];
+                    FxSource f;
+                    fx_split(p.x * unit, src_lim, f.hx, f.lx, f.fx);
+                    fx_split(p.y * unit, src_lim, f.hy, f.ly, f.fy);
+                    fx_split(p.z * unit, src_lim, f.hz, f.lz, f.fz);
+                    fx_split_charge(p.w * qs, f.qh, f.ql, f.fq);
+                    sm.fx[s] = f;
+                }
+                __syncthreads();
+            }
+            if (native || native_tiles > 0) {
+                --native_tiles;
+                if (field)
+                    tile64<true>(sm, buf, cnt, self_rel, skip_zero);
                 else
-                    tile64<true, 0>(b4, cnt, tx, self_rel, phi, g);
+                    tile64<false>(sm, buf, cnt, self_rel, skip_zero);
             } else {
-                if (skip == 2)
-                    tile64<false, 2>(b4, cnt, tx, self_rel, phi, g);
-                else
-                    tile64<false, 0>(b4, cnt, tx, self_rel, phi, g);
+                const double ps = rg.scale * exp2i(eq - 1022), fs = ps * rg.scale;
+                const int slow = field ? tile_fx<true>(sm, buf, cnt, tg, self_rel, skip_zero, ps, fs)
+                                       : tile_fx<false>(sm, buf, cnt, tg, self_rel, skip_zero, ps, fs);
+                native_tiles = 4 * slow > 3 * cnt ? 7 : 0;
             }
             __syncthreads();
             if (tid == 0 && k + 2 < ntile) issue(k + 2, buf);
@@ -639,7 +829,8 @@ __global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
 #pragma unroll
         for (int t = 0; t < kT64; ++t) {
             if (tidx[t] < 0) continue;
-            rec[tidx[t]] = make_double4_32a(phi[t], g[t][0], g[t][1], g[t][2]);
+            rec[tidx[t]] = make_double4_32a(sm.acc[t][0][tid], sm.acc[t][1][tid], sm.acc[t][2][tid],
+                                            sm.acc[t][3][tid]);
         }
         __syncthreads();
     }
@@ -767,7 +958,7 @@ int pair_targets_per_block(int precision, int variant)
 
 static size_t pair_smem(int precision, int variant)
 {
-    if (precision == HSMA_FP64) return 2 * kTile64 * sizeof(double4_32a);
+    if (precision == HSMA_FP64) return sizeof(FxShared);
     // staging: 2 buffers x (hi, lo); mode 1 adds the interleaved (hi, lo),
     // mode 2 the 4T double-float accumulators of every thread
     const size_t tile = (size_t)pair_targets_per_block(precision, variant);
@@ -801,6 +992,22 @@ int pair_max_ctas_per_sm(int precision, int variant)
     case 17: return occupancy_of(pair_fp32_kernel<3, 4, 1>, sm);
     default: return occupancy_of(pair_fp32_kernel<4, 4, 0>, sm);
     }
+}
+
+FxRange pair_fx_range(double r_src, double r_tgt)
+{
+    // the largest power of two with (r_src + r_tgt) scale <= 2: differences in
+    // units 2^-30 then fit 31 bits and a sign; the source limit one below its
+    // range leaves the targets theirs
+    FxRange g;
+    int e = 0;
+    const double r = r_src + r_tgt;
+    if (!(r_src > 0.0) || !(r_tgt > 0.0) || !std::isfinite(r)) return g;
+    if (std::frexp(r, &e) == 0.5) --e;  // r <= 2^e
+    if (std::abs(e) > 400) return g;
+    g.scale = std::ldexp(1.0, 1 - e);
+    g.src_lim = std::min(std::ceil(r_src * g.scale * 0x1p30), 2147483646.0) - 1.0;
+    return g;
 }
 
 // The dynamic shared-memory attribute is set by pair_max_ctas_per_sm, which
