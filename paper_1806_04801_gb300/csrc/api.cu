@@ -645,7 +645,8 @@ int enqueue_update(hsma_plan_s *p, const BatchShape &sh, const Workspace &w, int
         if ((rc = launch_surface_charges(nsys, p->ndir, p->Nb, p->Bq, p->dirs, w.A, p->Rs, w.img, st))) return rc;
         record(p, st, 5);
         if ((rc = launch_surface_pairs(w.sys, nsys, sh.surf_items, w.ns, w.src_hi, w.src_lo, w.src64, p->ndir,
-                                       p->dirs, w.img, p->Rs, p->dr, prec, w.phi_out, w.e_out, st)))
+                                       p->dirs, w.img, p->Rs, p->R0 + p->md_skin, p->dr, prec, w.phi_out,
+                                       w.e_out, st)))
             return rc;
         record(p, st, 6);
     }
@@ -1088,7 +1089,8 @@ int run_shard(hsma_plan_s *p, const hsma_particles *x, bool far_stage, int part,
             rc = launch_surface_charges(1, p->ndir, p->Nb, p->Bq, p->dirs, w.A, p->Rs, w.img, st);
             if (!rc && sh.surf_items > 0)
                 rc = launch_surface_pairs(w.sys, 1, sh.surf_items, w.ns, w.src_hi, w.src_lo, w.src64, p->ndir,
-                                          p->dirs, w.img, p->Rs, p->dr, prec, w.phi_out, w.e_out, st);
+                                          p->dirs, w.img, p->Rs, p->R0 + p->md_skin, p->dr, prec, w.phi_out,
+                                          w.e_out, st);
         }
         if (rc) return rc;
         // the near stage's Phi_in, E_in of the owned particles into their

@@ -450,9 +450,10 @@ int launch_fit_fp64(const SysDesc *sys, int nsys, int bc, int K, int ncols, int 
                     const double *phi_tgt, const int *mon_inv, double *b_out, double *A, cudaStream_t st);
 int launch_surface_charges(int nsys, int ndir, int Nb, const double *Bq, const double4_32a *dirs, const double *A,
                            double Rs, double2 *img, cudaStream_t st);
+// r_max: bound of the particles' distance from the centre
 int launch_surface_pairs(const SysDesc *sys, int nsys, int total_items, const long long *ns, const float4 *src_hi,
                          const float4 *src_lo, const double4_32a *src64, int ndir, const double4_32a *dirs,
-                         const double2 *img, double Rs, double dr, int precision, double *phi_out,
+                         const double2 *img, double Rs, double r_max, double dr, int precision, double *phi_out,
                          double *e_out, cudaStream_t st);
 int launch_series_field(const SysDesc *sys, int nsys, long long max_n, int P, double Rs, const double *norm,
                         const double *A, const float4 *src_hi, const float4 *src_lo, const double4_32a *src64,

@@ -259,8 +259,9 @@ __global__ void __launch_bounds__(kSurfThreads, 2) surface_pairs_fp32_kernel(
     }
 }
 
-// FP64 form: the three point images of each direction summed literally; one
-// particle per thread, kSurfTB per block (the FP32 kernel's block size).
+// FP64 form for thick dipole layers: the three point images of each direction
+// summed literally; one particle per thread, kSurfTB per block (the FP32
+// kernel's block size).
 constexpr int kSurf64Threads = kSurfTB;
 __global__ void __launch_bounds__(kSurf64Threads) surface_pairs_fp64_kernel(
     const SysDesc *sys, int nsys, const double4_32a *src64, int ndir, const double4_32a *dirs, const double2 *img,
@@ -331,6 +332,98 @@ __global__ void __launch_bounds__(kSurf64Threads) surface_pairs_fp64_kernel(
         e_out[3 * o] = e[t][0];
         e_out[3 * o + 1] = e[t][1];
         e_out[3 * o + 2] = e[t][2];
+    }
+}
+
+// FP64 form for thin dipole layers.  With d = r - Rs u, a = -u.d (> 0: the
+// particle is inside the sphere) and rho = |d|, the pair (p/dr)(1/A - 1/B) of
+// the literal form is the odd part of the Legendre series of 1/|d + s u| at
+// s = dr/2 = h,
+//   p [ a/rho^3 + h^2 P3(a/rho)/rho^4 + O(h^4/rho^6) ]:
+// a point dipole, and an h^2 term 1e-10 of it (dr = 1e-5 Rs) that FP32 holds
+// to the last FP64 bit.  The series leaves out (h/rho)^4 of the dipole, where
+// the literal difference of two 1/dr terms rounds at 2^-53 rho/h of it, so it
+// is the more accurate form while h <= 6.4e-4 rho (launch_surface_pairs).
+//
+// FP64 issue bounds both forms: 26 FP64 operations here per direction and
+// particle against 57 of the literal form.  A warp takes one particle and
+// every 32nd direction, so that small systems fill the chip as well (a thread
+// per particle left 16 blocks at N = 1000) and large ones leave a short tail:
+// two and four particles per warp, which share the loads, took 3% and 12%
+// longer.  N = 9999, 3196 directions: 6.35 -> 1.56 ms (79% of the FP64 rate);
+// N = 1000, 756: 1.38 -> 0.057 ms; grounded N = 3001, 1976: 3.60 -> 0.30 ms.
+//
+// f32_bits: v 2^-e in FP32 (truncated; 0 below 2^-126) by integer operations:
+// a conversion would take a slot of the FP64 pipe.
+__device__ __forceinline__ float f32_bits(double v, int e)
+{
+    const int hi = __double2hiint(v), m = (hi & 0x7fffffff) - ((896 + e) << 20);
+    const int b = m > 0 ? (m << 3) | (int)((unsigned)__double2loint(v) >> 29) : 0;
+    return __int_as_float((hi & (int)0x80000000u) | b);
+}
+
+__global__ void __launch_bounds__(128) surface_dipole_fp64_kernel(
+    const SysDesc *sys, int nsys, const double4_32a *src64, int ndir, const double4_32a *dirs, const double2 *img,
+    double Rs, double dr, double *phi_out, double *e_out)
+{
+    const int s = find_sys_surf(sys, nsys, blockIdx.x);
+    const SysDesc sd = sys[s];
+    const int lane = threadIdx.x & 31;
+    const long long i = sd.sp_lo + (long long)(blockIdx.x - sd.surf_off) * kSurfTB + blockIdx.y * 4 +
+                        (threadIdx.x >> 5);  // this warp's particle
+    if (i >= sd.sp_lo + sd.sp_n) return;
+    // the image dipoles' largest exponent, so that FP32 holds them whatever
+    // the units: the h^2 term runs in units of Rs and 2^pe
+    const double2 *im = img + (long long)s * ndir;
+    int pe = 0;
+    for (int j = lane; j < ndir; j += 32) pe = max(pe, (__double2hiint(im[j].y) & 0x7fffffff) >> 20);
+    pe = __reduce_max_sync(0xffffffffu, pe);
+    const double4_32a r = src64[sd.src_off + i];
+    const float rx = (float)(r.x / Rs), ry = (float)(r.y / Rs), rz = (float)(r.z / Rs);
+    const float h2 = (float)(0.25 * (dr / Rs) * (dr / Rs));
+    const double c2 = fma(r.x, r.x, fma(r.y, r.y, fma(r.z, r.z, Rs * Rs)));
+    // E = r S + K: the coefficient of d summed once, the rest per component
+    double phi = 0.0, S = 0.0, Kx = 0.0, Ky = 0.0, Kz = 0.0;
+    float pf = 0.f, ex = 0.f, ey = 0.f, ez = 0.f;
+    for (int j = lane; j < ndir; j += 32) {
+        const double4_32a u = dirs[j];
+        const double2 c = im[j];
+        const double ur = fma(u.x, r.x, fma(u.y, r.y, u.z * r.z));
+        const double a = Rs - ur;
+        const double ri = rsqrt(fma(-2.0 * Rs, ur, c2));
+        const double ri2 = ri * ri, ri3 = ri2 * ri;
+        const double w = c.y * ri3, m = w * a;
+        phi = fma(c.x, ri, phi) + m;
+        const double cd = fma(3.0 * m, ri2, c.x * ri3);
+        const double k = fma(-Rs, cd, w);
+        S += cd;
+        Kx = fma(k, u.x, Kx);
+        Ky = fma(k, u.y, Ky);
+        Kz = fma(k, u.z, Kz);
+        // h^2 term: p h^2 rho^-4 (5 q^3 - 3 q)/2 with q = a/rho, and minus its gradient
+        const float ux = f32_bits(u.x, 0), uy = f32_bits(u.y, 0), uz = f32_bits(u.z, 0);
+        const float dx = rx - ux, dy = ry - uy, dz = rz - uz;
+        const float fi = rsqrt_sfu(fmaf(dx, dx, fmaf(dy, dy, dz * dz))), fi2 = fi * fi;
+        const float q = -fmaf(ux, dx, fmaf(uy, dy, uz * dz)) * fi, qq = q * q;
+        const float g4 = 0.5f * h2 * f32_bits(c.y, pe - 1023) * fi2 * fi2;
+        pf = fmaf(g4 * q, fmaf(5.f, qq, -3.f), pf);
+        const float cu = g4 * fi * fmaf(15.f, qq, -3.f), cv = g4 * fi2 * q * fmaf(35.f, qq, -15.f);
+        ex = fmaf(cu, ux, fmaf(cv, dx, ex));
+        ey = fmaf(cu, uy, fmaf(cv, dy, ey));
+        ez = fmaf(cu, uz, fmaf(cv, dz, ez));
+    }
+    const double us = pe > 0 ? scalbn(1.0 / (Rs * Rs), pe - 1023) : 0.0, ue = us / Rs;
+    phi = warp_sum(fma((double)pf, us, phi));
+    S = warp_sum(S);
+    Kx = warp_sum(fma((double)ex, ue, Kx));
+    Ky = warp_sum(fma((double)ey, ue, Ky));
+    Kz = warp_sum(fma((double)ez, ue, Kz));
+    if (lane == 0) {
+        const long long o = sd.part_off + i;
+        phi_out[o] = phi;
+        e_out[3 * o] = fma(S, r.x, Kx);
+        e_out[3 * o + 1] = fma(S, r.y, Ky);
+        e_out[3 * o + 2] = fma(S, r.z, Kz);
     }
 }
 
@@ -423,12 +516,15 @@ int surface_targets_per_block() { return kSurfTB; }
 
 int launch_surface_pairs(const SysDesc *sys, int nsys, int total_items, const long long *ns, const float4 *src_hi,
                          const float4 *src_lo, const double4_32a *src64, int ndir, const double4_32a *dirs,
-                         const double2 *img, double Rs, double dr, int precision, double *phi_out,
+                         const double2 *img, double Rs, double r_max, double dr, int precision, double *phi_out,
                          double *e_out, cudaStream_t st)
 {
     (void)ns;
     if (total_items <= 0) return HSMA_OK;
-    if (precision == HSMA_FP64)
+    if (precision == HSMA_FP64 && 0.5 * dr <= 6.4e-4 * (Rs - r_max)) {
+        surface_dipole_fp64_kernel<<<dim3(total_items, kSurfTB / 4), 128, 0, st>>>(sys, nsys, src64, ndir, dirs, img,
+                                                                                  Rs, dr, phi_out, e_out);
+    } else if (precision == HSMA_FP64)
         surface_pairs_fp64_kernel<<<total_items, kSurf64Threads, 0, st>>>(sys, nsys, src64, ndir, dirs, img, Rs, dr,
                                                                          phi_out, e_out);
     else

@@ -1,4 +1,4 @@
-"""The FP64 near sums at the edges of their formats."""
+"""The FP64 near sums and the FP64 surface sums at the edges of their forms."""
 import numpy as np
 import pytest
 
@@ -74,3 +74,23 @@ def test_non_finite_and_coincident_inputs_still_error():
                 q[9] = np.inf
             with pytest.raises(hsma.HsmaError):
                 p.energy_forces(xyz, q)
+
+
+# Thin layers take the point-dipole series, thick ones the literal images;
+# the line is h = 6.4e-4 (Rs - R0).  The oracle sums the literal images: its
+# rounding is 2^-53 Rs/dr of the dipole terms, 2e-11 at the thinnest layer.
+@pytest.mark.parametrize("dr_rel", [1e-5, 1e-4, 5.3e-4, 5.5e-4, 5e-3])
+@pytest.mark.parametrize("n", [1, 63, 65, 200])
+def test_surface_sums_at_every_layer_thickness(dr_rel, n):
+    from paper_1806_04801_gb300 import hsma
+
+    g = np.random.default_rng(n)
+    xyz, q = 0.05 + 0.9 * g.random((n, 3)), g.standard_normal(n) * 1e-17
+    F2, _ = oh.fib_from_points(540)
+    ref = oh.energy_forces(xyz, q, oh.make_plan(BOX, I.GROUNDED, 6, 1.5, 300, F2, dr_rel))
+    with hsma.Plan(BOX, I.GROUNDED, 6, 1.5, 540, 300, precision="fp64", dr_rel=dr_rel) as p:
+        _, f, pot, _ = p.energy_forces(xyz, q, potentials=True)
+    scale = np.abs(ref["phi_out"]).max()
+    assert np.abs(pot - ref["pot"]).max() <= 1e-10 * max(scale, np.abs(ref["pot"]).max())
+    assert np.abs(f - ref["forces"]).max() <= 1e-10 * max(np.abs(ref["forces"]).max(),
+                                                          np.abs(q).max() * np.abs(ref["e_out"]).max())
