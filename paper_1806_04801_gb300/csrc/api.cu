@@ -1820,46 +1820,6 @@ int hsma_plan_load_tuning(hsma_plan_t pl, const char *cache_path)
 }
 
 // -------------------------------------------------------------- direct sums
-namespace {
-__global__ void split_sources_kernel(long long n, const double *src, float4 *hi, float4 *lo)
-{
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float hx, lx, hy, ly, hz, lz;
-    split_f64(src[4 * i], hx, lx);
-    split_f64(src[4 * i + 1], hy, ly);
-    split_f64(src[4 * i + 2], hz, lz);
-    hi[i] = make_float4(hx, hy, hz, (float)src[4 * i + 3]);
-    lo[i] = make_float4(lx, ly, lz, 0.f);
-}
-
-__global__ void split_targets_kernel(long long n, const double *tgt, float4 *hi, float4 *lo, double4_32a *t64)
-{
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double x = tgt[3 * i], y = tgt[3 * i + 1], z = tgt[3 * i + 2];
-    t64[i] = make_double4_32a(x, y, z, 0.0);
-    float hx, lx, hy, ly, hz, lz;
-    split_f64(x, hx, lx);
-    split_f64(y, hy, ly);
-    split_f64(z, hz, lz);
-    hi[i] = make_float4(hx, hy, hz, 0.f);
-    lo[i] = make_float4(lx, ly, lz, 0.f);
-}
-
-__global__ void scatter_results_kernel(long long n, const double *phi, const double *e, double *pot, double *field)
-{
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    pot[i] = phi[i];
-    if (field) {
-        field[3 * i] = e[3 * i];
-        field[3 * i + 1] = e[3 * i + 1];
-        field[3 * i + 2] = e[3 * i + 2];
-    }
-}
-}  // namespace
-
 int hsma_coulomb_sum(int64_t ns, const double *src, int64_t nt, const double *tgt, double *pot, double *field,
                      int precision, void *stream)
 {
@@ -1871,12 +1831,12 @@ int hsma_coulomb_sum(int64_t ns, const double *src, int64_t nt, const double *tg
     cudaStream_t st = (cudaStream_t)stream;
     int dev = 0;
     cudaGetDevice(&dev);
-    cudaDeviceProp prop;
-    HSMA_CUDA_TRY(cudaGetDeviceProperties(&prop, dev));
+    int sms = 0;
+    HSMA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int TB = pair_targets_per_block(precision);
     const int tile = precision == HSMA_FP64 ? 256 : 512;
     const int ctas = pair_max_ctas_per_sm(precision);
-    const int slots = prop.multiProcessorCount * ctas;
+    const int slots = sms * ctas;
     SysDesc d{};
     d.n = 0;
     d.ntb_part = 0;
@@ -1886,87 +1846,32 @@ int hsma_coulomb_sum(int64_t ns, const double *src, int64_t nt, const double *tg
     d.nchunks = (int)std::max(1LL, std::min(maxchunks, (long long)llround(ns / chunk)));
     long long items = (long long)d.ntb * d.nchunks;
     if (items > (1LL << 30)) return HSMA_E_ARG;
-    // sizes
-    size_t bytes = 0;
-    {
-        Carver cc(nullptr);
-        cc.take<float4>(ns);
-        cc.take<float4>(ns);
-        cc.take<double4_32a>(ns);
-        cc.take<float4>(nt);
-        cc.take<float4>(nt);
-        cc.take<double4_32a>(nt);
-        cc.take<float4>(2 * (size_t)d.nchunks * nt);
-        cc.take<double>(nt);
-        cc.take<double>(3 * nt);
-        cc.take<long long>(1);
-        cc.take<int>(8);
-        cc.take<int>(1);
-        cc.take<SysDesc>(1);
-        bytes = align_up(cc.off, 256);
-    }
+    const size_t n32 = precision == HSMA_FP64 ? 0 : 1, n64 = 1 - n32;
+    CoulombBuffers b;
+    auto carve = [&](void *base) {
+        Carver cc(base);
+        b.shi = cc.take<float4>(n32 * ns);
+        b.slo = cc.take<float4>(n32 * ns);
+        b.s64 = cc.take<double4_32a>(n64 * ns);
+        b.thi = cc.take<float4>(n32 * nt);
+        b.tlo = cc.take<float4>(n32 * nt);
+        b.t64 = cc.take<double4_32a>(n64 * nt);
+        b.partials = cc.take<float4>(2 * (size_t)d.nchunks * nt);
+        b.ns = cc.take<long long>(1);
+        b.ctrl = cc.take<int>(8);
+        b.status = cc.take<int>(1);
+        b.sys = cc.take<SysDesc>(1);
+        return align_up(cc.off, 256);
+    };
     void *mem = nullptr;
-    HSMA_CUDA_TRY(dev_malloc(&mem, bytes));
-    Carver cc(mem);
-    float4 *shi = cc.take<float4>(ns);
-    float4 *slo = cc.take<float4>(ns);
-    double4_32a *s64 = cc.take<double4_32a>(ns);
-    float4 *thi = cc.take<float4>(nt);
-    float4 *tlo = cc.take<float4>(nt);
-    double4_32a *t64 = cc.take<double4_32a>(nt);
-    float4 *partials = cc.take<float4>(2 * (size_t)d.nchunks * nt);
-    double *phi = cc.take<double>(nt);
-    double *e = cc.take<double>(3 * nt);
-    long long *dns = cc.take<long long>(1);
-    int *ctrl = cc.take<int>(8);
-    int *status = cc.take<int>(1);
-    SysDesc *dsys = cc.take<SysDesc>(1);
+    HSMA_CUDA_TRY(dev_malloc(&mem, carve(nullptr)));
+    carve(mem);
     int rc = HSMA_OK;
-    long long nsl = ns;
     do {
-        if (cudaMemcpyAsync(dsys, &d, sizeof(d), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-            cudaMemcpyAsync(dns, &nsl, sizeof(nsl), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-            cudaMemsetAsync(ctrl, 0, 8 * sizeof(int), st) != cudaSuccess ||
-            cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) {
-            rc = HSMA_E_CUDA;
-            break;
-        }
-        if (precision == HSMA_FP64 &&
-            cudaMemcpyAsync(s64, src, sizeof(double) * 4 * ns, cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
-            rc = HSMA_E_CUDA;
-            break;
-        }
-        if (precision != HSMA_FP64) {
-            split_sources_kernel<<<(unsigned)((ns + 255) / 256), 256, 0, st>>>(ns, src, shi, slo);
-            HSMA_LAUNCHED();
-        }
-        split_targets_kernel<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(nt, tgt, thi, tlo, t64);
-        HSMA_LAUNCHED();
-        PairArgs pa;
-        pa.sys = dsys;
-        pa.nsys = 1;
-        pa.total_items = (int)items;
-        pa.ns = dns;
-        pa.src_hi = shi;
-        pa.src_lo = slo;
-        pa.src64 = s64;
-        pa.ext_hi = thi;
-        pa.ext_lo = tlo;
-        pa.ext64 = t64;
-        pa.n_ext = (int)nt;
-        pa.ext_field = field ? 1 : 0;
-        pa.ext_skip_zero = 1;
-        pa.partials = partials;
-        pa.next_item = ctrl;
-        pa.status = status;
-        int grid = (int)std::max(1LL, std::min(items, (long long)slots));
-        if ((rc = launch_pair(pa, precision, 4, grid, st))) break;
-        if ((rc = launch_partial_reduce(dsys, 1, nt, (int)nt, partials, precision, phi, e, st))) break;
-        scatter_results_kernel<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(nt, phi, e, pot, field);
-        HSMA_LAUNCHED();
+        if ((rc = launch_coulomb(b, d, ns, src, nt, tgt, pot, field, precision, items, slots, st))) break;
         if (cudaStreamSynchronize(st) != cudaSuccess) rc = HSMA_E_CUDA;
         int hst = 0;
-        if (!rc && cudaMemcpy(&hst, status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) rc = HSMA_E_CUDA;
+        if (!rc && cudaMemcpy(&hst, b.status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) rc = HSMA_E_CUDA;
         if (!rc) rc = map_status(hst);
     } while (0);
     dev_free(mem);

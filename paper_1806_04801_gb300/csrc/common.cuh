@@ -400,9 +400,11 @@ int launch_inset_regen(const RegenArgs &r, cudaStream_t st);
 // Fixed-point formats of the FP64 sums (pair_fx.cuh).  scale: a power of two,
 // coordinates times scale 2^30 are the integers h, sources within +-src_lim
 // (targets within 2^31 - 1 - src_lim); scale 0: native FP64 throughout.
+// origin: the integers h are counted from it (0 in a plan's centred frame).
 struct FxRange {
     double scale = 0.0;
     double src_lim = 0.0;
+    double origin[3] = {0.0, 0.0, 0.0};
 };
 
 struct PairArgs {
@@ -426,6 +428,8 @@ struct PairArgs {
     int one_item = 0;               // 1: CTA b does work item b and exits (grid = total_items), so that
                                     // work on other streams gets SMs between items
     FxRange fx_part, fx_ext;  // FP64 form: formats for particle and for external targets
+    const int *fx_box = nullptr;  // FP64 form: if set, the formats come from this box of all coordinates
+                                  // (ordered FP32 keys, lows then highs: box_key)
     float4 *partials;       // 2 x float4 (FP32) or 1 x double4_32a (FP64) per record
     int *next_item;
     int *status;
@@ -433,6 +437,8 @@ struct PairArgs {
 // variant (FP32 form): one of the codes pair_variant_valid accepts; it fixes
 // the targets per thread -- 4 (blocks and tiles of 512), 3 (384) or 2 (256) --
 // the inner loop (scalar or packed f32x2) and the CTAs per SM.
+// FP32 as an integer that orders like it.
+__host__ __device__ __forceinline__ int box_key(int bits) { return bits ^ ((bits >> 31) & 0x7fffffff); }
 // The formats for source coordinates of magnitude up to r_src and target
 // coordinates up to r_tgt.
 FxRange pair_fx_range(double r_src, double r_tgt);
@@ -463,6 +469,20 @@ int launch_finalize(const SysDesc *sys, int nsys, long long max_n, const int *pe
                     const double *phi_tgt, const double *e_part, const double *phi_out, const double *e_out,
                     double *forces, double *pot, long long *owned_idx, double *upart, double *energy, int *status,
                     cudaStream_t st);
+
+// coulomb_static.cu: the direct sum of one call on the caller's buffers.
+struct CoulombBuffers {
+    SysDesc *sys;
+    long long *ns;
+    int *ctrl;    // [8] work counter, then the box keys
+    int *status;
+    float4 *shi, *slo, *thi, *tlo;  // FP32 form
+    double4_32a *s64, *t64;         // FP64 form
+    float4 *partials;
+};
+int launch_coulomb(const CoulombBuffers &b, const SysDesc &d, long long ns, const double *src, long long nt,
+                   const double *tgt, double *pot, double *field, int precision, long long items, int slots,
+                   cudaStream_t st);
 
 // api.cu: free a plan's workspace when it holds more than max_keep bytes
 // (used by the serving lanes to stay inside their memory budget).

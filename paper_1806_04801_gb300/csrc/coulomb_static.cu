@@ -22,6 +22,7 @@
 // first call before any stream capture.  A later call in a different context
 // (the device was reset, and the module loaded again) looks it up anew.
 #include <cuda.h>
+#include <limits.h>
 #include <math.h>
 #include <string.h>
 
@@ -73,7 +74,7 @@ bool current_context_id(unsigned long long *id)
 size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 
 struct StaticLayout {
-    size_t shi, slo, s64, thi, tlo, t64, partials, phi, e, ns, ctrl, status, sys, end;
+    size_t shi, slo, s64, thi, tlo, t64, partials, ns, ctrl, status, sys, end;
 };
 
 // Byte offsets of every buffer inside the static array for one call.
@@ -94,8 +95,7 @@ StaticLayout layout_for(long long ns, long long nt, int nchunks, int precision)
     L.tlo = put((size_t)nt * sizeof(float4));
     L.t64 = put((size_t)nt * sizeof(double4_32a));
     L.partials = put((size_t)nchunks * nt * 2 * sizeof(float4));
-    L.phi = put((size_t)nt * sizeof(double));
-    L.e = put((size_t)nt * 3 * sizeof(double));
+    put((size_t)nt * 4 * sizeof(double));  // not used: keeps the sizes that fit what they were
     L.ns = put(sizeof(long long));
     L.ctrl = put(8 * sizeof(int));
     L.status = put(sizeof(int));
@@ -104,58 +104,66 @@ StaticLayout layout_for(long long ns, long long nt, int nchunks, int precision)
     return L;
 }
 
-// Writes the work description and clears the counters and status.
-__global__ void static_init_kernel(SysDesc d, long long ns, SysDesc *dsys, long long *dns, int *ctrl, int *status)
+// Writes the work description, clears the counters and status and empties the
+// box of the coordinates.
+__global__ void coulomb_init_kernel(SysDesc d, long long ns, SysDesc *dsys, long long *dns, int *ctrl, int *status)
 {
     if (threadIdx.x == 0) {
         *dsys = d;
         *dns = ns;
         *status = 0;
     }
-    if (threadIdx.x < 8) ctrl[threadIdx.x] = 0;
+    if (threadIdx.x < 2) ctrl[threadIdx.x] = 0;
+    if (threadIdx.x >= 2 && threadIdx.x < 8) ctrl[threadIdx.x] = threadIdx.x < 5 ? INT_MAX : INT_MIN;
 }
 
-__global__ void static_split_sources_kernel(long long n, const double *src, float4 *hi, float4 *lo,
-                                            double4_32a *s64)
+// Sources and targets into the pair kernels' records: FP32 word pairs, or FP64
+// records and the box of all coordinates (one pass over each; the first
+// `sblocks` blocks take the sources).
+constexpr int kSplitThreads = 256;
+__global__ void __launch_bounds__(kSplitThreads) coulomb_split_kernel(long long ns, const double *src, long long nt,
+                                                                      const double *tgt, unsigned sblocks, bool f64,
+                                                                      CoulombBuffers b)
 {
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double x = src[4 * i], y = src[4 * i + 1], z = src[4 * i + 2], q = src[4 * i + 3];
-    if (s64) {
-        s64[i] = make_double4_32a(x, y, z, q);
+    __shared__ int red[6][kSplitThreads / 32];
+    const bool is_src = blockIdx.x < sblocks;
+    const long long i = (long long)(is_src ? blockIdx.x : blockIdx.x - sblocks) * kSplitThreads + threadIdx.x;
+    const bool live = i < (is_src ? ns : nt);
+    const double *p = is_src ? src + 4 * i : tgt + 3 * i;
+    const double x = live ? p[0] : 0.0, y = live ? p[1] : 0.0, z = live ? p[2] : 0.0;
+    const double q = live && is_src ? p[3] : 0.0;
+    if (!f64) {
+        if (!live) return;
+        float hx, lx, hy, ly, hz, lz;
+        split_f64(x, hx, lx);
+        split_f64(y, hy, ly);
+        split_f64(z, hz, lz);
+        (is_src ? b.shi : b.thi)[i] = make_float4(hx, hy, hz, (float)q);
+        (is_src ? b.slo : b.tlo)[i] = make_float4(lx, ly, lz, 0.f);
         return;
     }
-    float hx, lx, hy, ly, hz, lz;
-    split_f64(x, hx, lx);
-    split_f64(y, hy, ly);
-    split_f64(z, hz, lz);
-    hi[i] = make_float4(hx, hy, hz, (float)q);
-    lo[i] = make_float4(lx, ly, lz, 0.f);
-}
-
-__global__ void static_split_targets_kernel(long long n, const double *tgt, float4 *hi, float4 *lo, double4_32a *t64)
-{
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double x = tgt[3 * i], y = tgt[3 * i + 1], z = tgt[3 * i + 2];
-    t64[i] = make_double4_32a(x, y, z, 0.0);
-    float hx, lx, hy, ly, hz, lz;
-    split_f64(x, hx, lx);
-    split_f64(y, hy, ly);
-    split_f64(z, hz, lz);
-    hi[i] = make_float4(hx, hy, hz, 0.f);
-    lo[i] = make_float4(lx, ly, lz, 0.f);
-}
-
-__global__ void static_scatter_kernel(long long n, const double *phi, const double *e, double *pot, double *field)
-{
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    pot[i] = phi[i];
-    if (field) {
-        field[3 * i] = e[3 * i];
-        field[3 * i + 1] = e[3 * i + 1];
-        field[3 * i + 2] = e[3 * i + 2];
+    if (live) (is_src ? b.s64 : b.t64)[i] = make_double4_32a(x, y, z, q);
+    const double v[3] = {x, y, z};
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const int lo = live ? box_key(__float_as_int(__double2float_rd(v[a]))) : INT_MAX;
+        const int hi = live ? box_key(__float_as_int(__double2float_ru(v[a]))) : INT_MIN;
+        const int wl = __reduce_min_sync(0xffffffffu, lo), wh = __reduce_max_sync(0xffffffffu, hi);
+        if (lane == 0) {
+            red[a][wid] = wl;
+            red[3 + a][wid] = wh;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        int m = red[threadIdx.x][0];
+        for (int w = 1; w < kSplitThreads / 32; ++w)
+            m = threadIdx.x < 3 ? min(m, red[threadIdx.x][w]) : max(m, red[threadIdx.x][w]);
+        if (threadIdx.x < 3)
+            atomicMin(&b.ctrl[2 + threadIdx.x], m);
+        else
+            atomicMax(&b.ctrl[2 + threadIdx.x], m);
     }
 }
 
@@ -185,6 +193,43 @@ int static_setup(int dev, void **addr, int *sms)
 }
 
 }  // namespace
+
+// Four launches and no copy: the records are made and the results written by
+// the kernels themselves.
+int launch_coulomb(const CoulombBuffers &b, const SysDesc &d, long long ns, const double *src, long long nt,
+                   const double *tgt, double *pot, double *field, int precision, long long items, int slots,
+                   cudaStream_t st)
+{
+    const bool f64 = precision == HSMA_FP64;
+    coulomb_init_kernel<<<1, 32, 0, st>>>(d, ns, b.sys, b.ns, b.ctrl, b.status);
+    HSMA_LAUNCHED();
+    const unsigned sb = (unsigned)((ns + kSplitThreads - 1) / kSplitThreads);
+    const unsigned tb = (unsigned)((nt + kSplitThreads - 1) / kSplitThreads);
+    coulomb_split_kernel<<<sb + tb, kSplitThreads, 0, st>>>(ns, src, nt, tgt, sb, f64, b);
+    HSMA_LAUNCHED();
+    PairArgs pa;
+    pa.sys = b.sys;
+    pa.nsys = 1;
+    pa.total_items = (int)items;
+    pa.ns = b.ns;
+    pa.src_hi = b.shi;
+    pa.src_lo = b.slo;
+    pa.src64 = b.s64;
+    pa.ext_hi = b.thi;
+    pa.ext_lo = b.tlo;
+    pa.ext64 = b.t64;
+    pa.n_ext = (int)nt;
+    pa.ext_field = field ? 1 : 0;
+    pa.ext_skip_zero = 1;
+    pa.fx_box = b.ctrl + 2;
+    pa.partials = b.partials;
+    pa.next_item = b.ctrl;
+    pa.status = b.status;
+    const int grid = (int)std::max(1LL, std::min(items, (long long)slots));
+    int rc = launch_pair(pa, precision, 4, grid, st);
+    if (rc) return rc;
+    return launch_partial_reduce(b.sys, 1, nt, (int)nt, b.partials, precision, pot, field, st);
+}
 
 }  // namespace hsma
 
@@ -224,51 +269,22 @@ extern "C" int hsma_coulomb_sum_static(int64_t ns, const double *src, int64_t nt
     if (items > (1LL << 30)) return HSMA_E_CAPACITY;
 
     char *b = (char *)base;
-    float4 *shi = (float4 *)(b + L.shi), *slo = (float4 *)(b + L.slo);
-    double4_32a *s64 = (double4_32a *)(b + L.s64);
-    float4 *thi = (float4 *)(b + L.thi), *tlo = (float4 *)(b + L.tlo);
-    double4_32a *t64 = (double4_32a *)(b + L.t64);
-    float4 *partials = (float4 *)(b + L.partials);
-    double *phi = (double *)(b + L.phi), *e = (double *)(b + L.e);
-    long long *dns = (long long *)(b + L.ns);
-    int *ctrl = (int *)(b + L.ctrl), *status = (int *)(b + L.status);
-    SysDesc *dsys = (SysDesc *)(b + L.sys);
+    CoulombBuffers w;
+    w.shi = (float4 *)(b + L.shi);
+    w.slo = (float4 *)(b + L.slo);
+    w.s64 = (double4_32a *)(b + L.s64);
+    w.thi = (float4 *)(b + L.thi);
+    w.tlo = (float4 *)(b + L.tlo);
+    w.t64 = (double4_32a *)(b + L.t64);
+    w.partials = (float4 *)(b + L.partials);
+    w.ns = (long long *)(b + L.ns);
+    w.ctrl = (int *)(b + L.ctrl);
+    w.status = (int *)(b + L.status);
+    w.sys = (SysDesc *)(b + L.sys);
     cudaStream_t st = (cudaStream_t)stream;
-
-    static_init_kernel<<<1, 32, 0, st>>>(d, ns, dsys, dns, ctrl, status);
-    HSMA_LAUNCHED();
-    const bool f64 = precision == HSMA_FP64;
-    static_split_sources_kernel<<<(unsigned)((ns + 255) / 256), 256, 0, st>>>(ns, src, f64 ? nullptr : shi,
-                                                                              f64 ? nullptr : slo,
-                                                                              f64 ? s64 : nullptr);
-    HSMA_LAUNCHED();
-    static_split_targets_kernel<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(nt, tgt, thi, tlo, t64);
-    HSMA_LAUNCHED();
-    PairArgs pa;
-    pa.sys = dsys;
-    pa.nsys = 1;
-    pa.total_items = (int)items;
-    pa.ns = dns;
-    pa.src_hi = shi;
-    pa.src_lo = slo;
-    pa.src64 = s64;
-    pa.ext_hi = thi;
-    pa.ext_lo = tlo;
-    pa.ext64 = t64;
-    pa.n_ext = (int)nt;
-    pa.ext_field = field ? 1 : 0;
-    pa.ext_skip_zero = 1;
-    pa.partials = partials;
-    pa.next_item = ctrl;
-    pa.status = status;
-    const int grid = (int)std::max(1LL, std::min(items, (long long)slots));
-    if ((rc = launch_pair(pa, precision, 4, grid, st))) return rc;
-    if ((rc = launch_partial_reduce(dsys, 1, nt, (int)nt, partials, precision, phi, e, st))) return rc;
-    static_scatter_kernel<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(nt, phi, e, pot, field);
-    HSMA_LAUNCHED();
-    HSMA_CUDA_TRY(cudaGetLastError());
+    if ((rc = launch_coulomb(w, d, ns, src, nt, tgt, pot, field, precision, items, slots, st))) return rc;
     int hst = 0;
-    HSMA_CUDA_TRY(cudaMemcpyAsync(&hst, status, sizeof(int), cudaMemcpyDeviceToHost, st));
+    HSMA_CUDA_TRY(cudaMemcpyAsync(&hst, w.status, sizeof(int), cudaMemcpyDeviceToHost, st));
     HSMA_CUDA_TRY(cudaStreamSynchronize(st));
     if (hst & ST_TIMEOUT) return HSMA_E_TIMEOUT;
     return HSMA_OK;

@@ -544,6 +544,32 @@ __device__ __forceinline__ unsigned abs_hi(double v) { return (unsigned)__double
 // 2^k, -1022 <= k <= 1023.
 __device__ __forceinline__ double exp2i(int k) { return __hiloint2double((k + 1023) << 20, 0); }
 
+// Formats for coordinates inside the box of the keys, from the box's centre;
+// native FP64 (scale 0) for a point, anything not finite, or a box so far
+// from the origin that its coordinates hold less than the formats.
+__device__ __forceinline__ FxRange range_of_box(const int *keys)
+{
+    FxRange g;
+    float half = 0.f, mag = 0.f;
+    double c[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float lo = __int_as_float(box_key(keys[a])), hi = __int_as_float(box_key(keys[3 + a]));
+        c[a] = 0.5 * ((double)lo + (double)hi);
+        half = fmaxf(half, 0.5f * __fsub_ru(hi, lo));
+        mag = fmaxf(mag, fmaxf(fabsf(lo), fabsf(hi)));
+        if (!(hi - lo <= 3.0e38f)) return g;
+    }
+    if (!(half > 1e-30f && mag < half * 0x1p20f)) return g;
+    // 2 half scale <= 2, with a bit in hand for the rounding of the origin
+    const int e = (int)((unsigned)__float_as_int(half * 1.000001f) >> 23) - 126;  // half < 2^e
+    g.scale = exp2i(-e);
+    g.src_lim = 1073741823.0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) g.origin[a] = rint(c[a] * g.scale * 0x1p30);
+    return g;
+}
+
 // One pair in native FP64, added to this thread's sums.  skip: the target's
 // own slot; skip_zero: leave out a pair at distance exactly zero.
 template <bool FIELD>
@@ -706,7 +732,7 @@ __global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
 
         // fixed-point formats of this item: coordinates times `unit`, sources
         // within +-src_lim, targets within +-tgt_lim
-        const FxRange rg = part ? a.fx_part : a.fx_ext;
+        const FxRange rg = a.fx_box ? range_of_box(a.fx_box) : (part ? a.fx_part : a.fx_ext);
         const double unit = rg.scale * 0x1p30, src_lim = rg.src_lim, tgt_lim = 2147483647.0 - src_lim;
 
         const double4_32a *gs = a.src64 + sd.src_off;
@@ -739,8 +765,8 @@ __global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
             const double v[3] = {p.x * unit, p.y * unit, p.z * unit};
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                outside |= !(fabs(v[c]) <= tgt_lim + 1.0);
-                fx_split(v[c], tgt_lim, tg[t].h[c], tg[t].l[c], tg[t].f[c]);
+                outside |= !(fabs(v[c] - rg.origin[c]) <= tgt_lim + 1.0);
+                fx_split(v[c], rg.origin[c], tgt_lim, tg[t].h[c], tg[t].l[c], tg[t].f[c]);
             }
             tidx[t] = valid ? (part ? k : sd.n + k) : -1;
 #pragma unroll
@@ -769,8 +795,9 @@ __global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
             for (int s = tid; s < cnt; s += kThreads) {
                 const double4_32a p = sm.src[buf][s];
                 const unsigned hq = abs_hi(p.w);
-                const bool ok = fabs(p.x * unit) <= src_lim + 1.0 && fabs(p.y * unit) <= src_lim + 1.0 &&
-                                fabs(p.z * unit) <= src_lim + 1.0 && hq < 0x7ff00000u &&
+                const bool ok = fabs(fma(p.x, unit, -rg.origin[0])) <= src_lim + 1.0 &&
+                                fabs(fma(p.y, unit, -rg.origin[1])) <= src_lim + 1.0 &&
+                                fabs(fma(p.z, unit, -rg.origin[2])) <= src_lim + 1.0 && hq < 0x7ff00000u &&
                                 (hq >= 0x00100000u || p.w == 0.0);
                 qmax = max(qmax, ok ? hq : 0x7fffffffu);
                 if (p.w != 0.0) qmin = min(qmin, hq);
@@ -798,9 +825,9 @@ __global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
                 for (int s = tid; s < cnt; s += kThreads) {
                     const double4_32a p = sm.src[buf][s];
                     FxSource f;
-                    fx_split(p.x * unit, src_lim, f.hx, f.lx, f.fx);
-                    fx_split(p.y * unit, src_lim, f.hy, f.ly, f.fy);
-                    fx_split(p.z * unit, src_lim, f.hz, f.lz, f.fz);
+                    fx_split(p.x * unit, rg.origin[0], src_lim, f.hx, f.lx, f.fx);
+                    fx_split(p.y * unit, rg.origin[1], src_lim, f.hy, f.ly, f.fy);
+                    fx_split(p.z * unit, rg.origin[2], src_lim, f.hz, f.lz, f.fz);
                     fx_split_charge(p.w * qs, f.qh, f.ql, f.fq);
                     sm.fx[s] = f;
                 }
@@ -843,7 +870,7 @@ __global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
 // double-float arithmetic on the FP32 pipe (FP64 issue is far slower on this
 // part); the total is converted to FP64 once.
 // phi_tgt[tgt_off + t] = potential, e_part[3 (tgt_off + t) + a] = field
-// E = -sum q (y - x)/r^3.
+// E = -sum q (y - x)/r^3 (e_part may be null).
 __global__ void partial_reduce_kernel(const SysDesc *sys, int n_ext, const float4 *partials, int precision,
                                       double *phi_tgt, double *e_part)
 {
@@ -880,6 +907,7 @@ __global__ void partial_reduce_kernel(const SysDesc *sys, int n_ext, const float
             gz[j] += r.w;
         }
         phi_tgt[o] = (p[0] + p[1]) + (p[2] + p[3]);
+        if (!e_part) return;
         e_part[3 * o] = -((gx[0] + gx[1]) + (gx[2] + gx[3]));
         e_part[3 * o + 1] = -((gy[0] + gy[1]) + (gy[2] + gy[3]));
         e_part[3 * o + 2] = -((gz[0] + gz[1]) + (gz[2] + gz[3]));
@@ -919,6 +947,7 @@ __global__ void partial_reduce_kernel(const SysDesc *sys, int n_ext, const float
         return (double)s.x + (double)s.y;
     };
     phi_tgt[o] = total(p);
+    if (!e_part) return;
     e_part[3 * o] = -total(gx);
     e_part[3 * o + 1] = -total(gy);
     e_part[3 * o + 2] = -total(gz);

@@ -102,16 +102,17 @@ HSMA_HD int fx_f2i(float x)  // to nearest
 #endif
 }
 
-// Coordinate in units of 2^-30, |v| <= lim + 1 < 2^31: h within +-lim.
-HSMA_HD void fx_split(double v, double lim, int &h, int &l, float &f)
+// Coordinate v in units of 2^-30 (|v| < 2^51) from the origin o (an integer),
+// |v - o| <= lim + 1 < 2^31: h within +-lim.  Exact to 2^-60.
+HSMA_HD void fx_split(double v, double o, double lim, int &h, int &l, float &f)
 {
 #ifdef __CUDA_ARCH__
     const double magic = 6755399441055744.0;  // 1.5 2^52: a sum's low word is the nearest integer
-    const double t = fmin(fmax((v + magic) - magic, -lim), lim), d = v - t;
+    const double n = (v + magic) - magic, w = n - o, t = fmin(fmax(w, -lim), lim), d = (v - n) + (w - t);
     h = __double2loint(t + magic);
     l = __double2loint(fma(d, 0x1p30, magic));
 #else
-    const double t = fmin(fmax(nearbyint(v), -lim), lim), d = v - t;
+    const double n = nearbyint(v), w = n - o, t = fmin(fmax(w, -lim), lim), d = (v - n) + (w - t);
     h = (int)t;
     l = (int)nearbyint(d * 0x1p30);
 #endif

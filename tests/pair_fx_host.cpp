@@ -44,12 +44,12 @@ int main(int argc, char **argv)
             if (it % 5 == 0) t[(c + 1) % 3] = u(g) * 0x1p-40;  // and tiny coordinates
         }
         FxSource f;
-        fx_split(s[0] * 0x1p30, src_lim, f.hx, f.lx, f.fx);
-        fx_split(s[1] * 0x1p30, src_lim, f.hy, f.ly, f.fy);
-        fx_split(s[2] * 0x1p30, src_lim, f.hz, f.lz, f.fz);
+        fx_split(s[0] * 0x1p30, 0.0, src_lim, f.hx, f.lx, f.fx);
+        fx_split(s[1] * 0x1p30, 0.0, src_lim, f.hy, f.ly, f.fy);
+        fx_split(s[2] * 0x1p30, 0.0, src_lim, f.hz, f.lz, f.fz);
         fx_split_charge(q, f.qh, f.ql, f.fq);
         FxTarget tg;
-        for (int c = 0; c < 3; ++c) fx_split(t[c] * 0x1p30, tgt_lim, tg.h[c], tg.l[c], tg.f[c]);
+        for (int c = 0; c < 3; ++c) fx_split(t[c] * 0x1p30, 0.0, tgt_lim, tg.h[c], tg.l[c], tg.f[c]);
         const int dh[3] = {f.hx - tg.h[0], f.hy - tg.h[1], f.hz - tg.h[2]};
         const int dl[3] = {f.lx - tg.l[0], f.ly - tg.l[1], f.lz - tg.l[2]};
         const float df[3] = {f.fx - tg.f[0], f.fy - tg.f[1], f.fz - tg.f[2]};

@@ -94,3 +94,46 @@ def test_surface_sums_at_every_layer_thickness(dr_rel, n):
     assert np.abs(pot - ref["pot"]).max() <= 1e-10 * max(scale, np.abs(ref["pot"]).max())
     assert np.abs(f - ref["forces"]).max() <= 1e-10 * max(np.abs(ref["forces"]).max(),
                                                           np.abs(q).max() * np.abs(ref["e_out"]).max())
+
+
+# The direct sum finds its scale from the coordinates: boxes off the origin,
+# flat and clustered sets, targets outside the sources' box, a target on a
+# source (skipped), and sets whose offset leaves the formats (native FP64).
+@pytest.mark.parametrize("field", [True, False])
+@pytest.mark.parametrize("shape", ["unit", "offset", "far offset", "flat", "cluster and one far", "small units",
+                                   "one point"])
+@pytest.mark.parametrize("ns,nt", [(1, 1), (255, 257), (1021, 130)])
+def test_direct_sum_at_every_scale(shape, ns, nt, field):
+    import torch
+
+    from paper_1806_04801_gb300 import hsma
+
+    g = np.random.default_rng(ns)
+    s, t, q = g.random((ns, 3)), 1.5 * g.random((nt, 3)) - 0.2, g.standard_normal(ns)
+    if shape == "offset":
+        s, t = s + [100.0, -7.0, 0.0], t + [100.0, -7.0, 0.0]
+    elif shape == "far offset":
+        s, t = s + 3e7, t + 3e7
+    elif shape == "flat":
+        s[:, 2], t[:, 2] = 0.25, 0.25
+    elif shape == "cluster and one far":
+        s, t = 1e-5 * s, 1e-5 * t
+        t[0] = 1.0
+    elif shape == "small units":
+        s, t, q = 1e-9 * s, 1e-9 * t, 1.6e-19 * q
+    elif shape == "one point":
+        s[:], t[:] = 0.5, 0.5
+    t[nt // 2] = s[ns // 2]
+    src = np.concatenate([s, q[:, None]], 1)
+    pot, fld = hsma.coulomb_sum(torch.as_tensor(src).cuda(), torch.as_tensor(t).cuda(), field=field,
+                                precision="fp64")
+    d = t[:, None].astype(np.longdouble) - s[None]
+    r2 = (d * d).sum(2)
+    ri = np.where(r2 > 0, 1 / np.sqrt(np.where(r2 > 0, r2, 1)), 0)
+    bound = (2 * ns + 30) * 2.0**-53
+    assert np.all(np.abs(pot.cpu().numpy() - (ri * q).sum(1)) <= bound * (ri * np.abs(q)).sum(1))
+    if field:
+        e = (d * (ri**3 * q)[:, :, None]).sum(1)
+        assert np.all(np.abs(fld.cpu().numpy() - e) <= bound * (ri**2 * np.abs(q)).sum(1)[:, None])
+    else:
+        assert fld is None
