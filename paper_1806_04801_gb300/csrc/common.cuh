@@ -403,7 +403,7 @@ int launch_inset_regen(const RegenArgs &r, cudaStream_t st);
 // origin: the integers h are counted from it (0 in a plan's centred frame).
 struct FxRange {
     double scale = 0.0;
-    double src_lim = 0.0;
+    int src_lim = 0;
     double origin[3] = {0.0, 0.0, 0.0};
 };
 

@@ -39,7 +39,7 @@ constexpr int kThreads = 128;
 // FP32 form: T targets per thread (T = 2, 3 or 4, by variant); a block of
 // 128 T targets is exactly one in-set tile of 128 T sources, so a particle
 // block's box is its tile's box.
-constexpr int kT64 = 2;
+constexpr int kT64 = 1;
 constexpr int kTB64 = kThreads * kT64;
 constexpr int kTile64 = 256;
 constexpr int kFoldFx = 16;             // FxSums::gf fold interval (sources)
@@ -515,20 +515,24 @@ __global__ void __launch_bounds__(kThreads, MINB) pair_fp32_kernel(PairArgs a)
 // ------------------------------------------------------------ FP64 tiles
 // The FP64 sums run on the integer and FP32 pipes (pair_fx.cuh has the
 // arithmetic and the reason); pairs outside its formats take native FP64.
-// A CTA turns each staged tile into fixed point once (36 FP64 operations per
-// source for 256 targets) with the charges scaled by the tile's largest, and
-// sums it for two targets per thread; the tile's integer sums go to FP64
-// accumulators in shared memory.  Near pairs are a few in a thousand, but
-// some lane has one in 1-3% of a warp's steps; they use the otherwise idle
-// FP64 pipe while other warps go on (14% busy), so a larger near radius would
-// cost little and a smaller one would cost the field's precision.
+// A CTA turns each staged tile into fixed point once (by integer operations:
+// 36 FP64 ones per source cost 3-10%), with the charges scaled by the tile's
+// largest, and sums it for one target per thread; the tile's integer sums go
+// to FP64 accumulators in shared memory.  Two targets per thread share the
+// loads of a source, but blocks of 128 targets spread better: 0.24 against
+// 0.32 ms at N = 1000, 1.60 against 1.80 (grounded, N = 3001), 11.1 against
+// 11.0 at N = 9999.  Near pairs are a few in a thousand, but some lane has one
+// in 1-3% of a warp's steps; they use the otherwise idle FP64 pipe while other
+// warps go on (14% busy), so a larger near radius would cost little and a
+// smaller one would cost the field's precision.
 // Bound by the FMA-heavy pipe, which issues the 32 x 32 multiplies (78% of
-// its active cycles; ALU 44%, issue slots 64%).  Measured: near-sum phase of
-// N = 9999 (1.96e9 pairs) 61.3 -> 11.0 ms, 3.2e10 -> 1.78e11 pairs/s; N = 1000
-// 1.30 -> 0.32 ms; grounded N = 3001 9.4 -> 1.8 ms.  Error against quad
+// its active cycles; ALU 44%, issue slots 64%); keeping the 64-bit additions
+// apart from the multiplies was 7% slower.  Measured: near-sum phase of
+// N = 9999 (1.96e9 pairs) 61.3 -> 11.1 ms, 3.2e10 -> 1.77e11 pairs/s; N = 1000
+// 1.30 -> 0.24 ms; grounded N = 3001 9.4 -> 1.6 ms.  Error against quad
 // precision (N = 300..4000, both boundaries, three charge patterns): field
-// 1.9e-16..8.2e-16 of its norm against 4.7e-16..1.7e-15 before, potential
-// 1.3e-16..3.9e-15 against 3.5e-16..5.2e-15.
+// 1.6e-16..8.0e-16 of its norm against 4.7e-16..1.7e-15 before, potential
+// 1.5e-16..3.9e-15 against 3.5e-16..5.2e-15.
 struct FxShared {
     double4_32a src[2][kTile64];       // staged sources (bulk copies land here)
     FxSource fx[kTile64];              // the tile being summed, in fixed point
@@ -564,7 +568,7 @@ __device__ __forceinline__ FxRange range_of_box(const int *keys)
     // 2 half scale <= 2, with a bit in hand for the rounding of the origin
     const int e = (int)((unsigned)__float_as_int(half * 1.000001f) >> 23) - 126;  // half < 2^e
     g.scale = exp2i(-e);
-    g.src_lim = 1073741823.0;
+    g.src_lim = 1073741823;
 #pragma unroll
     for (int a = 0; a < 3; ++a) g.origin[a] = rint(c[a] * g.scale * 0x1p30);
     return g;
@@ -698,7 +702,7 @@ __device__ __forceinline__ int tile_fx(FxShared &sm, int buf, int cnt, const FxT
     return __reduce_max_sync(0xffffffffu, slow);
 }
 
-__global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
+__global__ void __launch_bounds__(kThreads, 5) pair_fp64_kernel(PairArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem64[];
     FxShared &sm = *reinterpret_cast<FxShared *>(smem64);
@@ -733,7 +737,12 @@ __global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
         // fixed-point formats of this item: coordinates times `unit`, sources
         // within +-src_lim, targets within +-tgt_lim
         const FxRange rg = a.fx_box ? range_of_box(a.fx_box) : (part ? a.fx_part : a.fx_ext);
-        const double unit = rg.scale * 0x1p30, src_lim = rg.src_lim, tgt_lim = 2147483647.0 - src_lim;
+        const int kx = 60 + (__double2hiint(rg.scale) >> 20) - 1023;  // coordinates 2^kx: units of l
+        const int src_lim = rg.src_lim, tgt_lim = 2147483647 - src_lim;
+        auto split = [&](double v, int c, int lim, int &h, int &l, float &f) {
+            if (a.fx_box) return fx_split_from(v * rg.scale * 0x1p30, rg.origin[c], lim, h, l, f);
+            return fx_split(fx_fixed(v, kx), lim, h, l, f) && fx_fits(v, kx);
+        };
 
         const double4_32a *gs = a.src64 + sd.src_off;
         const int ntile = t1 - t0;
@@ -762,17 +771,14 @@ __global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
             sm.tgt[t][0][tid] = p.x;
             sm.tgt[t][1][tid] = p.y;
             sm.tgt[t][2][tid] = p.z;
-            const double v[3] = {p.x * unit, p.y * unit, p.z * unit};
+            const double v[3] = {p.x, p.y, p.z};
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                outside |= !(fabs(v[c] - rg.origin[c]) <= tgt_lim + 1.0);
-                fx_split(v[c], rg.origin[c], tgt_lim, tg[t].h[c], tg[t].l[c], tg[t].f[c]);
-            }
+            for (int c = 0; c < 3; ++c) outside |= !split(v[c], c, tgt_lim, tg[t].h[c], tg[t].l[c], tg[t].f[c]);
             tidx[t] = valid ? (part ? k : sd.n + k) : -1;
 #pragma unroll
             for (int c = 0; c < 4; ++c) sm.acc[t][c][tid] = 0.0;
         }
-        const bool blk_native = __syncthreads_or(outside || !(unit > 0.0));
+        const bool blk_native = __syncthreads_or(outside || !(rg.scale > 0.0));
         int native_tiles = 0;  // this warp's next tiles go native: the last one held mostly near pairs
 
         for (int k = 0; k < ntile; ++k) {
@@ -790,15 +796,17 @@ __global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
                 const long long o = part && tidx[t] >= 0 ? tidx[t] - s0 : -1;
                 self_rel[t] = o >= 0 && o < kTile64 ? (int)o : -1;
             }
-            // charge range of the tile; 0x7fffffff marks what the formats do not hold
+            // charge range of the tile; 0x7fffffff marks what the formats do not
+            // hold.  The coordinates are converted on the way.
             unsigned qmax = 0u, qmin = 0x7fffffffu;
             for (int s = tid; s < cnt; s += kThreads) {
                 const double4_32a p = sm.src[buf][s];
+                FxSource &f = sm.fx[s];
                 const unsigned hq = abs_hi(p.w);
-                const bool ok = fabs(fma(p.x, unit, -rg.origin[0])) <= src_lim + 1.0 &&
-                                fabs(fma(p.y, unit, -rg.origin[1])) <= src_lim + 1.0 &&
-                                fabs(fma(p.z, unit, -rg.origin[2])) <= src_lim + 1.0 && hq < 0x7ff00000u &&
-                                (hq >= 0x00100000u || p.w == 0.0);
+                bool ok = hq < 0x7ff00000u && (hq >= 0x00100000u || p.w == 0.0);
+                ok = split(p.x, 0, src_lim, f.hx, f.lx, f.fx) && ok;
+                ok = split(p.y, 1, src_lim, f.hy, f.ly, f.fy) && ok;
+                ok = split(p.z, 2, src_lim, f.hz, f.lz, f.fz) && ok;
                 qmax = max(qmax, ok ? hq : 0x7fffffffu);
                 if (p.w != 0.0) qmin = min(qmin, hq);
             }
@@ -821,15 +829,9 @@ __global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
             const bool native =
                 blk_native || eq > 1923 || eq < 123 || (qmax != 0u && (int)(qmin >> 20) < eq - 20);
             if (!native) {
-                const double qs = exp2i(1022 - eq);
                 for (int s = tid; s < cnt; s += kThreads) {
-                    const double4_32a p = sm.src[buf][s];
-                    FxSource f;
-                    fx_split(p.x * unit, rg.origin[0], src_lim, f.hx, f.lx, f.fx);
-                    fx_split(p.y * unit, rg.origin[1], src_lim, f.hy, f.ly, f.fy);
-                    fx_split(p.z * unit, rg.origin[2], src_lim, f.hz, f.lz, f.fz);
-                    fx_split_charge(p.w * qs, f.qh, f.ql, f.fq);
-                    sm.fx[s] = f;
+                    fx_split_charge(fx_fixed(sm.src[buf][s].w, 63 + 1022 - eq), sm.fx[s].qh, sm.fx[s].ql,
+                                    sm.fx[s].fq);
                 }
                 __syncthreads();
             }
@@ -1035,7 +1037,7 @@ FxRange pair_fx_range(double r_src, double r_tgt)
     if (std::frexp(r, &e) == 0.5) --e;  // r <= 2^e
     if (std::abs(e) > 400) return g;
     g.scale = std::ldexp(1.0, 1 - e);
-    g.src_lim = std::min(std::ceil(r_src * g.scale * 0x1p30), 2147483646.0) - 1.0;
+    g.src_lim = (int)(std::min(std::ceil(r_src * g.scale * 0x1p30), 2147483646.0) - 1.0);
     return g;
 }
 

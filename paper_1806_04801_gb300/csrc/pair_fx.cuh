@@ -29,6 +29,7 @@
 
 #include <math.h>
 #include <stdint.h>
+#include <string.h>
 
 #ifdef __CUDACC__
 #define HSMA_HD __host__ __device__ __forceinline__
@@ -102,30 +103,67 @@ HSMA_HD int fx_f2i(float x)  // to nearest
 #endif
 }
 
-// Coordinate v in units of 2^-30 (|v| < 2^51) from the origin o (an integer),
-// |v - o| <= lim + 1 < 2^31: h within +-lim.  Exact to 2^-60.
-HSMA_HD void fx_split(double v, double o, double lim, int &h, int &l, float &f)
+HSMA_HD uint64_t fx_bits(double v)
+{
+#ifdef __CUDA_ARCH__
+    return (uint64_t)__double_as_longlong(v);
+#else
+    uint64_t b;
+    memcpy(&b, &v, sizeof b);
+    return b;
+#endif
+}
+
+// v 2^k rounded to an integer, by integer operations (a conversion through
+// the FP64 pipe costs as much as 64 of these); |v 2^k| < 2^63.
+HSMA_HD int64_t fx_fixed(double v, int k)
+{
+    const uint64_t b = fx_bits(v);
+    const int e = (int)(b >> 52) & 0x7ff, sh = (e > 0 ? e : 1) - 1075 + k;
+    const uint64_t m = (b & 0xfffffffffffffull) | (e > 0 ? 0x10000000000000ull : 0ull);
+    const uint64_t r = sh >= 0 ? m << sh : (sh > -64 ? ((m >> (-sh - 1)) + 1) >> 1 : 0ull);
+    return (int64_t)b < 0 ? -(int64_t)r : (int64_t)r;
+}
+
+// Whether |v 2^k| < 2^62 (no for a NaN).
+HSMA_HD bool fx_fits(double v, int k) { return ((int)(fx_bits(v) >> 52) & 0x7ff) <= 1084 - k; }
+
+// Coordinate X in units of 2^-60: h within +-lim; whether it lies there.
+HSMA_HD bool fx_split(int64_t X, int lim, int &h, int &l, float &f)
+{
+    const int64_t n = (X + 0x20000000LL) >> 30;
+    h = (int)(n < -lim ? -lim : (n > lim ? lim : n));
+    const int64_t d = X - ((int64_t)h << 30);
+    l = (int)d;
+    f = (float)l * 0x1p-30f;
+    return d <= 0x40000000LL && d >= -0x40000000LL;
+}
+
+// The same from an origin o (an integer in units 2^-30) that may be far off,
+// v in units of 2^-30, |v| < 2^51: exact, with FP64 operations.
+HSMA_HD bool fx_split_from(double v, double o, int lim, int &h, int &l, float &f)
 {
 #ifdef __CUDA_ARCH__
     const double magic = 6755399441055744.0;  // 1.5 2^52: a sum's low word is the nearest integer
-    const double n = (v + magic) - magic, w = n - o, t = fmin(fmax(w, -lim), lim), d = (v - n) + (w - t);
+    const double n = (v + magic) - magic, w = n - o, t = fmin(fmax(w, -(double)lim), (double)lim),
+                 d = (v - n) + (w - t);
     h = __double2loint(t + magic);
     l = __double2loint(fma(d, 0x1p30, magic));
 #else
-    const double n = nearbyint(v), w = n - o, t = fmin(fmax(w, -lim), lim), d = (v - n) + (w - t);
+    const double n = nearbyint(v), w = n - o, t = fmin(fmax(w, -(double)lim), (double)lim), d = (v - n) + (w - t);
     h = (int)t;
     l = (int)nearbyint(d * 0x1p30);
 #endif
     f = (float)d;
+    return fabs(d) <= 1.0;
 }
 
-// Charge, |v| < 1.
-HSMA_HD void fx_split_charge(double v, int &h, uint32_t &l, float &f)
+// Charge X in units of 2^-63, |q| < 1.
+HSMA_HD void fx_split_charge(int64_t X, int &h, uint32_t &l, float &f)
 {
-    const double t = v * 0x1p31, d = floor(t);
-    h = (int)d;
-    l = (uint32_t)((t - d) * 0x1p32);
-    f = (float)v;
+    h = (int)(X >> 32);
+    l = (uint32_t)X;
+    f = (float)X * 0x1p-63f;
 }
 
 // dh, dl: source minus target.  The distance^2 in units 2^-60.

@@ -19,7 +19,7 @@ int main(int argc, char **argv)
     const int mode = atoi(argv[1]), count = atoi(argv[2]);
     std::mt19937_64 g(atoi(argv[3]));
     std::uniform_real_distribution<double> u(-1.0, 1.0);
-    const double src_lim = 1.5 * 0x1p30 - 1.0, tgt_lim = 0x1p29;
+    const int src_lim = (3 << 29) - 1, tgt_lim = 1 << 29;
     ld wp = 0, wf = 0, we = 0;
     for (int it = 0; it < count; ++it) {
         double t[3], s[3], q = u(g);
@@ -44,12 +44,23 @@ int main(int argc, char **argv)
             if (it % 5 == 0) t[(c + 1) % 3] = u(g) * 0x1p-40;  // and tiny coordinates
         }
         FxSource f;
-        fx_split(s[0] * 0x1p30, 0.0, src_lim, f.hx, f.lx, f.fx);
-        fx_split(s[1] * 0x1p30, 0.0, src_lim, f.hy, f.ly, f.fy);
-        fx_split(s[2] * 0x1p30, 0.0, src_lim, f.hz, f.lz, f.fz);
-        fx_split_charge(q, f.qh, f.ql, f.fq);
+        bool in = fx_split(fx_fixed(s[0], 60), src_lim, f.hx, f.lx, f.fx);
+        in = fx_split(fx_fixed(s[1], 60), src_lim, f.hy, f.ly, f.fy) && in;
+        in = fx_split(fx_fixed(s[2], 60), src_lim, f.hz, f.lz, f.fz) && in;
+        fx_split_charge(fx_fixed(q, 63), f.qh, f.ql, f.fq);
         FxTarget tg;
-        for (int c = 0; c < 3; ++c) fx_split(t[c] * 0x1p30, 0.0, tgt_lim, tg.h[c], tg.l[c], tg.f[c]);
+        for (int c = 0; c < 3; ++c) {
+            in = fx_split(fx_fixed(t[c], 60), tgt_lim, tg.h[c], tg.l[c], tg.f[c]) && in;
+            int h, l;  // the form with an origin gives the same words
+            float fl;
+            in = fx_split_from(t[c] * 0x1p30 + 0x1p40, 0x1p40, tgt_lim, h, l, fl) && in;
+            if (std::abs(t[c]) > 0x1p-10 && std::abs(h - tg.h[c]) > 1) in = false;
+        }
+        if (!in || fx_fits(4.0, 60) ||
+            !fx_fits(3.9, 60) || fx_fits(NAN, 60)) {
+            printf("range\n");
+            return 1;
+        }
         const int dh[3] = {f.hx - tg.h[0], f.hy - tg.h[1], f.hz - tg.h[2]};
         const int dl[3] = {f.lx - tg.l[0], f.ly - tg.l[1], f.lz - tg.l[2]};
         const float df[3] = {f.fx - tg.f[0], f.fy - tg.f[1], f.fz - tg.f[2]};
