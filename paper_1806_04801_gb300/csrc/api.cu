@@ -301,7 +301,7 @@ void shape_batch(const hsma_plan_s *p, int nsys, const long long *n, int precisi
     sh->variant = pair_variant_valid(tu.pair_variant) ? tu.pair_variant : 4;
     const int TB = pair_targets_per_block(precision, sh->variant);
     const int STB = surface_targets_per_block();
-    const int tile = TB;
+    const int tile = pair_sources_per_tile(precision, sh->variant);
     const double vsphere = 4.0 / 3.0 * kPi * p->Rs * p->Rs * p->Rs;
     const double vbox = p->L[0] * p->L[1] * p->L[2];
     const int slots = p->num_sms * tuned_ctas(p, precision, sh->variant);

@@ -445,6 +445,7 @@ FxRange pair_fx_range(double r_src, double r_tgt);
 int launch_pair(const PairArgs &a, int precision, int variant, int grid, cudaStream_t st);
 bool pair_variant_valid(int variant);
 int pair_targets_per_block(int precision, int variant = 4);
+int pair_sources_per_tile(int precision, int variant = 4);
 int pair_max_ctas_per_sm(int precision, int variant = 4);
 int launch_partial_reduce(const SysDesc *sys, int nsys, long long max_tgt, int n_ext, const float4 *partials,
                           int precision, double *phi_tgt, double *e_part, cudaStream_t st);
