@@ -129,6 +129,7 @@ struct hsma_plan_s {
     std::vector<int> mon_perm;
     double *Mrow = nullptr, *Mp = nullptr, *Bq = nullptr, *norm = nullptr;
     double4_32a *dirs = nullptr;
+    float4 *dirs32 = nullptr;                              // the directions in FP32
     int4 *shifts = nullptr;
     void *tc_hi = nullptr, *tc_lo = nullptr;
     void *tc_mdf = nullptr;  // M (K x n_cols) as FP32 word pairs, for the refinement residual
@@ -642,10 +643,12 @@ int enqueue_update(hsma_plan_s *p, const BatchShape &sh, const Workspace &w, int
         record(p, st, 6);
     } else {
         // (d) surface images and their sums at the particles
-        if ((rc = launch_surface_charges(nsys, p->ndir, p->Nb, p->Bq, p->dirs, w.A, p->Rs, w.img, st))) return rc;
+        if ((rc = launch_surface_charges(nsys, p->ndir, p->Nb, p->Bq, p->dirs, w.A, p->Rs, prec != HSMA_FP64,
+                                         w.img, st)))
+            return rc;
         record(p, st, 5);
-        if ((rc = launch_surface_pairs(w.sys, nsys, sh.surf_items, w.ns, w.src_hi, w.src_lo, w.src64, p->ndir,
-                                       p->dirs, w.img, p->Rs, p->R0 + p->md_skin, p->dr, prec, w.phi_out,
+        if ((rc = launch_surface_pairs(w.sys, nsys, sh.surf_items, w.src_hi, w.src_lo, w.src64, p->ndir,
+                                       p->dirs, p->dirs32, w.img, p->Rs, p->R0 + p->md_skin, p->dr, prec, w.phi_out,
                                        w.e_out, st)))
             return rc;
         record(p, st, 6);
@@ -1086,10 +1089,10 @@ int run_shard(hsma_plan_s *p, const hsma_particles *x, bool far_stage, int part,
             rc = launch_series_field(w.sys, 1, std::max<long long>(cnt, 1), p->P, p->Rs, p->norm, w.A, w.src_hi,
                                      w.src_lo, w.src64, w.phi_out, w.e_out, st);
         } else {
-            rc = launch_surface_charges(1, p->ndir, p->Nb, p->Bq, p->dirs, w.A, p->Rs, w.img, st);
+            rc = launch_surface_charges(1, p->ndir, p->Nb, p->Bq, p->dirs, w.A, p->Rs, prec != HSMA_FP64, w.img, st);
             if (!rc && sh.surf_items > 0)
-                rc = launch_surface_pairs(w.sys, 1, sh.surf_items, w.ns, w.src_hi, w.src_lo, w.src64, p->ndir,
-                                          p->dirs, w.img, p->Rs, p->R0 + p->md_skin, p->dr, prec, w.phi_out,
+                rc = launch_surface_pairs(w.sys, 1, sh.surf_items, w.src_hi, w.src_lo, w.src64, p->ndir,
+                                          p->dirs, p->dirs32, w.img, p->Rs, p->R0 + p->md_skin, p->dr, prec, w.phi_out,
                                           w.e_out, st);
         }
         if (rc) return rc;
@@ -1348,6 +1351,7 @@ int hsma_plan(hsma_plan_t *out, const double box[3], int bc, int p, double R, in
         pl->Mrow = c.take<double>((size_t)K * ncols);
         pl->Mp = c.take<double>((size_t)ncols * K);
         pl->dirs = c.take<double4_32a>(ndir);
+        pl->dirs32 = c.take<float4>(ndir);
         pl->Bq = c.take<double>((size_t)ndir * Nb);
         pl->norm = c.take<double>(Nb);
         pl->shifts = c.take<int4>(sh.size());
@@ -1416,6 +1420,7 @@ int hsma_plan(hsma_plan_t *out, const double box[3], int bc, int p, double R, in
             break;
         if ((rc = build_pseudo_inverse(K, ncols, Mcol, pl->Mp, &cond, &rank_ok, st))) break;
         if ((rc = launch_quadrature(F2, F1, R, pl->dirs, st))) break;
+        if ((rc = launch_directions_fp32(ndir, pl->dirs, pl->dirs32, st))) break;
         // basis at Rs u_j == basis of the unit vector u_j with unit radius
         if ((rc = launch_basis(p, 1.0, ndir, (const double *)pl->dirs, 4, pl->Bq, Nb, st))) break;
         if ((rc = prepare_tc_operands(K, ncols, pl->Mp, pl->Mrow, pl->tc_hi, pl->tc_lo, pl->tc_mdf, st))) break;

@@ -20,25 +20,40 @@ namespace {
 
 constexpr double kPi = 3.14159265358979323846;
 
-__global__ void fit_fp64_kernel(const SysDesc *sys, int bc, int K, int ncols, int Nb, const double *Mp,
-                                const double *phi_tgt, const int *mon_inv, double *b_out, double *A)
+// A = M+ b, a row per S of a block's eight warps (S = 8: one system's few rows
+// over many SMs -- p = 10, K = 1500 has 120 rows, 15 blocks of eight and 47
+// dependent rounds each before; S = 1: batches).  The S partial sums are added
+// in warp order.
+template <int S>
+__global__ void __launch_bounds__(256) fit_fp64_kernel(const SysDesc *sys, int bc, int K, int ncols, int Nb,
+                                                       const double *Mp, const double *phi_tgt, const int *mon_inv,
+                                                       double *b_out, double *A)
 {
+    __shared__ double red[8];
     const SysDesc sd = sys[blockIdx.y];
     const double *ph = phi_tgt + sd.tgt_off + sd.n;  // monitoring targets
     const int drop = (bc == HSMA_BC_PERIODIC) ? 1 : 0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int c = blockIdx.x * (blockDim.x >> 5) + warp;
+    const int c = blockIdx.x * (8 / S) + warp / S;
     if (blockIdx.x == 0) {
         for (int i = threadIdx.x; i < K; i += blockDim.x)
             b_out[(long long)blockIdx.y * K + i] = rhs_at(ph, mon_inv, K, i, drop != 0);
         if (drop && threadIdx.x == 0) A[(long long)blockIdx.y * Nb] = 0.0;
     }
-    if (c >= ncols) return;
-    const double *row = Mp + (long long)c * K;
     double s = 0.0;
-    for (int i = lane; i < K; i += 32) s += row[i] * rhs_at(ph, mon_inv, K, i, drop != 0);
+    if (c < ncols) {
+        const double *row = Mp + (long long)c * K;
+        for (int i = (warp % S) * 32 + lane; i < K; i += 32 * S) s += row[i] * rhs_at(ph, mon_inv, K, i, drop != 0);
+    }
     s = warp_sum(s);
-    if (lane == 0) A[(long long)blockIdx.y * Nb + c + drop] = s;
+    if (S > 1) {
+        if (lane == 0) red[warp] = s;
+        __syncthreads();
+        if (warp % S != 0) return;
+        s = 0.0;
+        for (int k = 0; k < S; ++k) s += red[warp + k];
+    }
+    if (lane == 0 && c < ncols) A[(long long)blockIdx.y * Nb + c + drop] = s;
 }
 
 __device__ __forceinline__ int degree_of(int k)
@@ -49,26 +64,46 @@ __device__ __forceinline__ int degree_of(int k)
     return n;
 }
 
-// One warp per (system, direction).
-__global__ void surface_charges_kernel(int ndir, int Nb, const double *Bq, const double4_32a *dirs, const double *A,
-                                       double Rs, double2 *img)
+// Sigma and dipole images of kChargeDirs directions of a system per block, a
+// warp per direction at a time; A and n A_nm staged once per block, so that an
+// element takes two FP64 operations (FP64 issue bounds batches: 0.33 -> 0.18 ms
+// for 32 systems at p = 10).  img: double2 (Q_sigma, p), or with f32 the same
+// pairs as float2 for the FP32 surface sums, whose blocks then stage them
+// without a conversion each.
+constexpr int kChargeDirs = 16;
+__global__ void __launch_bounds__(256) surface_charges_kernel(int ndir, int Nb, const double *Bq,
+                                                              const double4_32a *dirs, const double *A, double Rs,
+                                                              int f32, double2 *img)
 {
-    const int lane = threadIdx.x & 31;
-    const int d = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (d >= ndir) return;
+    extern __shared__ double2 an[];  // (A_nm, n A_nm)
     const double *a = A + (long long)blockIdx.y * Nb;
-    const double *row = Bq + (long long)d * Nb;
-    double phi = 0.0, sig = 0.0;
-    for (int k = lane; k < Nb; k += 32) {
-        double v = row[k] * a[k];
-        phi += v;
-        sig += degree_of(k) * v;
+    for (int k = threadIdx.x; k < Nb; k += blockDim.x) {
+        const double v = a[k];
+        an[k] = make_double2(v, degree_of(k) * v);
     }
-    phi = warp_sum(phi);
-    sig = warp_sum(sig);
-    if (lane == 0) {
-        double w = dirs[d].w;
-        img[(long long)blockIdx.y * ndir + d] = make_double2(w * sig / (Rs * 4.0 * kPi), w * phi / (4.0 * kPi));
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const int hi = min(ndir, (int)(blockIdx.x + 1) * kChargeDirs);
+    for (int d = blockIdx.x * kChargeDirs + (threadIdx.x >> 5); d < hi; d += 8) {
+        const double *row = Bq + (long long)d * Nb;
+        double phi = 0.0, sig = 0.0;
+#pragma unroll 4
+        for (int k = lane; k < Nb; k += 32) {
+            const double v = row[k];
+            const double2 c = an[k];
+            phi = fma(v, c.x, phi);
+            sig = fma(v, c.y, sig);
+        }
+        phi = warp_sum(phi);
+        sig = warp_sum(sig);
+        if (lane == 0) {
+            const double w = dirs[d].w, q = w * sig / (Rs * 4.0 * kPi), p = w * phi / (4.0 * kPi);
+            const long long o = (long long)blockIdx.y * ndir + d;
+            if (f32)
+                reinterpret_cast<float2 *>(img)[o] = make_float2((float)q, (float)p);
+            else
+                img[o] = make_double2(q, p);
+        }
     }
 }
 
@@ -96,7 +131,8 @@ __device__ __forceinline__ int find_sys_surf(const SysDesc *sys, int nsys, int i
     return lo;
 }
 
-// FP32 form.  For direction u with d = r - Rs u, h = dr/2, a = u.d:
+// FP32 form for thick layers.  For direction u with d = r - Rs u, h = dr/2,
+// a = u.d:
 //   sigma image:  Q/|d|, field Q d/|d|^3
 //   dipole pair:  (p/dr)(1/A - 1/B) with A = |d + h u|, B = |d - h u|
 //                 = -2 p a / (A B (A + B))                  (no cancellation)
@@ -112,8 +148,8 @@ __device__ __forceinline__ int find_sys_surf(const SysDesc *sys, int nsys, int i
 constexpr int kSurfPairs = kSurfTile / kSurfSplit / 2;  // direction pairs per group per tile
 
 __global__ void __launch_bounds__(kSurfThreads, 2) surface_pairs_fp32_kernel(
-    const SysDesc *sys, int nsys, const float4 *src_hi, const float4 *src_lo, int ndir, const double4_32a *dirs,
-    const double2 *img, float Rs, float h, double *phi_out, double *e_out)
+    const SysDesc *sys, int nsys, const float4 *src_hi, const float4 *src_lo, int ndir, const float4 *dirs,
+    const float2 *img, float Rs, float h, double *phi_out, double *e_out)
 {
     __shared__ float4 sx[kSurfSplit][kSurfPairs], sy[kSurfSplit][kSurfPairs], sz[kSurfSplit][kSurfPairs];
     __shared__ float2 red[kSurfSplit - 1][kSurfT][4][kSurfGroup];  // partial sums of groups 1..
@@ -147,7 +183,7 @@ __global__ void __launch_bounds__(kSurfThreads, 2) surface_pairs_fp32_kernel(
         phi[t] = make_float2(0.f, 0.f);
         e[t][0] = e[t][1] = e[t][2] = make_float2(0.f, 0.f);
     }
-    const double2 *im = img + (long long)s * ndir;
+    const float2 *im = img + (long long)s * ndir;
     float *fx = reinterpret_cast<float *>(&sx[0][0]), *fy = reinterpret_cast<float *>(&sy[0][0]);
     float *fz = reinterpret_cast<float *>(&sz[0][0]);
     for (int d0 = 0; d0 < ndir; d0 += kSurfTile) {
@@ -156,14 +192,13 @@ __global__ void __launch_bounds__(kSurfThreads, 2) surface_pairs_fp32_kernel(
         for (int j = threadIdx.x; j < kSurfTile; j += kSurfThreads) {
             float ux = 1.f, uy = 0.f, uz = 0.f, Q = 0.f, pw = 0.f;
             if (j < cnt) {
-                const double4_32a u = dirs[d0 + j];
-                const double2 c = im[d0 + j];
-                const bool live = u.w > 0.0;
-                ux = (float)u.x;
-                uy = (float)u.y;
-                uz = (float)u.z;
-                Q = live ? (float)c.x : 0.f;
-                pw = live ? (float)c.y : 0.f;
+                const float4 u = dirs[d0 + j];
+                const float2 c = im[d0 + j];
+                ux = u.x;
+                uy = u.y;
+                uz = u.z;
+                Q = u.w > 0.f ? c.x : 0.f;
+                pw = u.w > 0.f ? c.y : 0.f;
             }
             const int g = j % kSurfSplit, k = j / kSurfSplit, kp = k >> 1, ln = k & 1;
             const int base = (g * kSurfPairs + kp) * 4;
@@ -252,6 +287,157 @@ __global__ void __launch_bounds__(kSurfThreads, 2) surface_pairs_fp32_kernel(
         }
         if (idx[t] < 0) continue;
         long long o = sd.part_off + idx[t];
+        phi_out[o] = (double)phi[t].x + (double)phi[t].y;
+        e_out[3 * o] = (double)e[t][0].x + (double)e[t][0].y;
+        e_out[3 * o + 1] = (double)e[t][1].x + (double)e[t][1].y;
+        e_out[3 * o + 2] = (double)e[t][2].x + (double)e[t][2].y;
+    }
+}
+
+// FP32 form for thin layers: the dipole pair as its Legendre series (see the
+// FP64 form below), with d, a = -u.d and rho = |d|:
+//   potential  Q/rho + m (1 + k0),                     m = p a/rho^3
+//   field      (Q/rho^3 + (3 m/rho^2)(1 + k2)) d + (p/rho^3)(1 + k1) u
+//   k0 = s (5 q^2 - 3), k1 = s (15 q^2 - 3), k2 = s (35 q^2 - 15)/3,
+//   s = h^2/(2 rho^2), q = a/rho;
+// H2 = false leaves the k's out where they are below the FP32 rounding
+// (12 s < 6e-9), and the next terms, (h/rho)^4, are below it up to h = 5e-3 rho.
+// 24 (with the k's 36) FP32 lane operations and one SFU result per direction
+// and particle against about 50 and four of the literal form above.
+//
+// A block of 256 threads is G direction groups of 256/G lanes with T particles
+// each; the directions of a staged tile go round the groups, two per packed
+// instruction.  G = 8, T = 2 (64 particles a block) for large systems;
+// G = 32, T = 1 (8 particles) where that leaves SMs without a block.  The
+// FP32 directions come from the plan and the images in FP32 from
+// surface_charges: staging converted seven FP64 values per direction and
+// block before, at two per SM and clock.
+// Measured: N = 100000, 3196 directions 0.533 -> 0.293 ms; N = 4000 0.066 ->
+// 0.029; N = 500, 1976 directions 0.043 -> 0.014; with the k's, grounded
+// N = 20000 0.102 -> 0.078; 32 boxes of 500..50000 0.731 -> 0.397.
+template <int G, int T, bool H2>
+__global__ void __launch_bounds__(256) surface_dipole_fp32_kernel(const SysDesc *sys, int nsys, const float4 *src_hi,
+                                                                  const float4 *src_lo, int ndir, const float4 *dirs,
+                                                                  const float2 *img, float Rs, float hh,
+                                                                  double *phi_out, double *e_out)
+{
+    constexpr int L = 256 / G, kPairs = kSurfTile / 2;
+    // direction pairs: (ux, ux', uy, uy'), (uz, uz', Q, Q'), (p, p')
+    __shared__ float4 sx[kPairs], sy[kPairs];
+    __shared__ float2 sz[kPairs];
+    __shared__ float2 red[G - 1][T][4][L];  // partial sums of groups 1..
+    const int s = find_sys_surf(sys, nsys, blockIdx.x);
+    const SysDesc sd = sys[s];
+    const int gl = threadIdx.x % L, grp = threadIdx.x / L;
+    const long long hi = sd.sp_lo + sd.sp_n;
+    const long long i0 = sd.sp_lo + (long long)(blockIdx.x - sd.surf_off) * kSurfTB + (long long)blockIdx.y * L * T;
+    if (i0 >= hi) return;
+    float2 RX[T], RY[T], RZ[T];  // particle position, both lanes
+    long long idx[T];
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+        const long long i = i0 + t * L + gl;
+        idx[t] = i < hi ? i : -1;
+        const float4 a = src_hi[sd.src_off + min(i, hi - 1)], b = src_lo[sd.src_off + min(i, hi - 1)];
+        const float rx = a.x + b.x, ry = a.y + b.y, rz = a.z + b.z;
+        RX[t] = make_float2(rx, rx);
+        RY[t] = make_float2(ry, ry);
+        RZ[t] = make_float2(rz, rz);
+    }
+    const float2 NRS = make_float2(-Rs, -Rs), M1 = make_float2(-1.f, -1.f), C3 = make_float2(3.f, 3.f);
+    float2 phi[T], e[T][3];
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+        phi[t] = make_float2(0.f, 0.f);
+        e[t][0] = e[t][1] = e[t][2] = make_float2(0.f, 0.f);
+    }
+    const float2 *im = img + (long long)s * ndir;
+    for (int d0 = 0; d0 < ndir; d0 += kSurfTile) {
+        __syncthreads();
+        for (int j = threadIdx.x; j < kPairs; j += 256) {
+            // beyond the last direction: one without images
+            const int a = d0 + 2 * j, b = a + 1;
+            const float4 u = a < ndir ? dirs[a] : make_float4(1.f, 0.f, 0.f, 0.f);
+            const float4 v = b < ndir ? dirs[b] : make_float4(1.f, 0.f, 0.f, 0.f);
+            const float2 c = a < ndir ? im[a] : make_float2(0.f, 0.f), f = b < ndir ? im[b] : make_float2(0.f, 0.f);
+            sx[j] = make_float4(u.x, v.x, u.y, v.y);
+            sy[j] = make_float4(u.z, v.z, c.x, f.x);
+            sz[j] = make_float2(c.y, f.y);
+        }
+        __syncthreads();
+        const int npairs = min(kPairs, (ndir - d0 + 1) >> 1);
+        float2 pa[T], ea[T][3];
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+            pa[t] = make_float2(0.f, 0.f);
+            ea[t][0] = ea[t][1] = ea[t][2] = make_float2(0.f, 0.f);
+        }
+#pragma unroll 2
+        for (int kp = grp; kp < npairs; kp += G) {
+            const float4 X = sx[kp], Y = sy[kp];
+            const float2 p = sz[kp];
+            const float2 ux = make_float2(X.x, X.y), uy = make_float2(X.z, X.w);
+            const float2 uz = make_float2(Y.x, Y.y), Q = make_float2(Y.z, Y.w);
+#pragma unroll
+            for (int t = 0; t < T; ++t) {
+                const float2 dx = __ffma2_rn(NRS, ux, RX[t]);
+                const float2 dy = __ffma2_rn(NRS, uy, RY[t]);
+                const float2 dz = __ffma2_rn(NRS, uz, RZ[t]);
+                const float2 dd = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+                const float2 na = __ffma2_rn(ux, dx, __ffma2_rn(uy, dy, __fmul2_rn(uz, dz)));  // -a
+                const float2 ri = make_float2(rsqrt_sfu(dd.x), rsqrt_sfu(dd.y));
+                const float2 ri2 = __fmul2_rn(ri, ri), ri3 = __fmul2_rn(ri2, ri);
+                float2 w = __fmul2_rn(p, ri3);
+                float2 m = __fmul2_rn(__fmul2_rn(w, na), M1);
+                float2 m3 = __fmul2_rn(m, ri2);
+                if (H2) {
+                    const float2 qq = __fmul2_rn(__fmul2_rn(na, na), ri2);
+                    const float2 sc = __fmul2_rn(make_float2(hh, hh), ri2);
+                    const float2 k0 = __ffma2_rn(make_float2(5.f, 5.f), qq, make_float2(-3.f, -3.f));
+                    const float2 k1 = __ffma2_rn(make_float2(15.f, 15.f), qq, make_float2(-3.f, -3.f));
+                    const float2 k2 = __ffma2_rn(make_float2(35.f / 3.f, 35.f / 3.f), qq, make_float2(-5.f, -5.f));
+                    m = __ffma2_rn(m, __fmul2_rn(sc, k0), m);
+                    w = __ffma2_rn(w, __fmul2_rn(sc, k1), w);
+                    m3 = __ffma2_rn(m3, __fmul2_rn(sc, k2), m3);
+                }
+                pa[t] = __fadd2_rn(__ffma2_rn(Q, ri, pa[t]), m);
+                const float2 cd = __ffma2_rn(C3, m3, __fmul2_rn(Q, ri3));
+                ea[t][0] = __ffma2_rn(cd, dx, __ffma2_rn(w, ux, ea[t][0]));
+                ea[t][1] = __ffma2_rn(cd, dy, __ffma2_rn(w, uy, ea[t][1]));
+                ea[t][2] = __ffma2_rn(cd, dz, __ffma2_rn(w, uz, ea[t][2]));
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+            phi[t] = df_add(phi[t], pa[t].x + pa[t].y);
+            e[t][0] = df_add(e[t][0], ea[t][0].x + ea[t][0].y);
+            e[t][1] = df_add(e[t][1], ea[t][1].x + ea[t][1].y);
+            e[t][2] = df_add(e[t][2], ea[t][2].x + ea[t][2].y);
+        }
+    }
+    // add the groups' partial sums in group order
+    if (grp > 0) {
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+            red[grp - 1][t][0][gl] = phi[t];
+            red[grp - 1][t][1][gl] = e[t][0];
+            red[grp - 1][t][2][gl] = e[t][1];
+            red[grp - 1][t][3][gl] = e[t][2];
+        }
+    }
+    __syncthreads();
+    if (grp > 0) return;
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+#pragma unroll 7
+        for (int g2 = 0; g2 < G - 1; ++g2) {
+            phi[t] = df_add_df(phi[t], red[g2][t][0][gl]);
+            e[t][0] = df_add_df(e[t][0], red[g2][t][1][gl]);
+            e[t][1] = df_add_df(e[t][1], red[g2][t][2][gl]);
+            e[t][2] = df_add_df(e[t][2], red[g2][t][3][gl]);
+        }
+        if (idx[t] < 0) continue;
+        const long long o = sd.part_off + idx[t];
         phi_out[o] = (double)phi[t].x + (double)phi[t].y;
         e_out[3 * o] = (double)e[t][0].x + (double)e[t][0].y;
         e_out[3 * o + 1] = (double)e[t][1].x + (double)e[t][1].y;
@@ -435,7 +621,7 @@ __global__ void __launch_bounds__(128) surface_dipole_fp64_kernel(
 // owned_idx == nullptr: outputs at the caller's indices; otherwise (one
 // system) output j is particle sp_lo + j and owned_idx[j] its caller index.
 constexpr int kFinalThreads = 256;
-constexpr int kFinal = 2048;
+constexpr int kFinal = 256;  // one particle per thread: 2048 left one or two blocks to systems of a few thousand
 
 __global__ void __launch_bounds__(kFinalThreads) finalize_kernel(const SysDesc *sys, const int *perm, const double *q,
                                                                  const double *phi_tgt, const double *e_part,
@@ -477,15 +663,17 @@ __global__ void __launch_bounds__(kFinalThreads) finalize_kernel(const SysDesc *
     if (threadIdx.x == 0) upart[(long long)s * nb_max + blockIdx.x] = u;
 }
 
-// U = 1/2 sum of the block partials, in block order (of the owned range).
+// U = 1/2 sum of the block partials (of the owned range): a warp, each lane
+// every 32nd partial in order, then a fixed tree.
 __global__ void energy_kernel(const SysDesc *sys, const double *upart, int nb_max, double *energy, int *status)
 {
     const int s = blockIdx.x;
-    if (threadIdx.x != 0) return;
     const SysDesc sd = sys[s];
     const int nb = (int)((sd.sp_n + kFinal - 1) / kFinal);
     double u = 0.0;
-    for (int b = 0; b < nb; ++b) u += upart[(long long)s * nb_max + b];
+    for (int b = threadIdx.x; b < nb; b += 32) u += upart[(long long)s * nb_max + b];
+    u = warp_sum(u);
+    if (threadIdx.x != 0) return;
     energy[s] = 0.5 * u;
     if (!isfinite(u)) atomicOr(&status[s], ST_COINCIDENT);
 }
@@ -495,18 +683,21 @@ __global__ void energy_kernel(const SysDesc *sys, const double *upart, int nb_ma
 int launch_fit_fp64(const SysDesc *sys, int nsys, int bc, int K, int ncols, int Nb, const double *Mp,
                     const double *phi_tgt, const int *mon_inv, double *b_out, double *A, cudaStream_t st)
 {
-    dim3 grid((ncols + 7) / 8, nsys);
-    fit_fp64_kernel<<<grid, 256, 0, st>>>(sys, bc, K, ncols, Nb, Mp, phi_tgt, mon_inv, b_out, A);
+    if ((long long)ncols * nsys <= 1216)  // a block per row fills the chip
+        fit_fp64_kernel<8><<<dim3(ncols, nsys), 256, 0, st>>>(sys, bc, K, ncols, Nb, Mp, phi_tgt, mon_inv, b_out, A);
+    else
+        fit_fp64_kernel<1><<<dim3((ncols + 7) / 8, nsys), 256, 0, st>>>(sys, bc, K, ncols, Nb, Mp, phi_tgt, mon_inv,
+                                                                       b_out, A);
     HSMA_LAUNCHED();
     HSMA_CUDA_TRY(cudaGetLastError());
     return HSMA_OK;
 }
 
 int launch_surface_charges(int nsys, int ndir, int Nb, const double *Bq, const double4_32a *dirs, const double *A,
-                           double Rs, double2 *img, cudaStream_t st)
+                           double Rs, bool f32, double2 *img, cudaStream_t st)
 {
-    dim3 grid((ndir + 7) / 8, nsys);
-    surface_charges_kernel<<<grid, 256, 0, st>>>(ndir, Nb, Bq, dirs, A, Rs, img);
+    dim3 grid((ndir + kChargeDirs - 1) / kChargeDirs, nsys);
+    surface_charges_kernel<<<grid, 256, Nb * sizeof(double2), st>>>(ndir, Nb, Bq, dirs, A, Rs, f32 ? 1 : 0, img);
     HSMA_LAUNCHED();
     HSMA_CUDA_TRY(cudaGetLastError());
     return HSMA_OK;
@@ -514,22 +705,52 @@ int launch_surface_charges(int nsys, int ndir, int Nb, const double *Bq, const d
 
 int surface_targets_per_block() { return kSurfTB; }
 
-int launch_surface_pairs(const SysDesc *sys, int nsys, int total_items, const long long *ns, const float4 *src_hi,
-                         const float4 *src_lo, const double4_32a *src64, int ndir, const double4_32a *dirs,
+int launch_surface_pairs(const SysDesc *sys, int nsys, int total_items, const float4 *src_hi, const float4 *src_lo,
+                         const double4_32a *src64, int ndir, const double4_32a *dirs, const float4 *dirs32,
                          const double2 *img, double Rs, double r_max, double dr, int precision, double *phi_out,
                          double *e_out, cudaStream_t st)
 {
-    (void)ns;
     if (total_items <= 0) return HSMA_OK;
-    if (precision == HSMA_FP64 && 0.5 * dr <= 6.4e-4 * (Rs - r_max)) {
+    const double h = 0.5 * dr, rho = Rs - r_max;  // rho: a lower bound
+    const float2 *img32 = reinterpret_cast<const float2 *>(img);
+    if (precision == HSMA_FP64 && h <= 6.4e-4 * rho) {
         surface_dipole_fp64_kernel<<<dim3(total_items, kSurfTB / 4), 128, 0, st>>>(sys, nsys, src64, ndir, dirs, img,
                                                                                   Rs, dr, phi_out, e_out);
-    } else if (precision == HSMA_FP64)
+    } else if (precision == HSMA_FP64) {
         surface_pairs_fp64_kernel<<<total_items, kSurf64Threads, 0, st>>>(sys, nsys, src64, ndir, dirs, img, Rs, dr,
                                                                          phi_out, e_out);
-    else
-        surface_pairs_fp32_kernel<<<total_items, kSurfThreads, 0, st>>>(
-            sys, nsys, src_hi, src_lo, ndir, dirs, img, (float)Rs, (float)(0.5 * dr), phi_out, e_out);
+    } else if (h <= 5e-3 * rho) {
+        auto launch = [&](auto kernel, int particles) {
+            kernel<<<dim3(total_items, kSurfTB / particles), 256, 0, st>>>(sys, nsys, src_hi, src_lo, ndir, dirs32,
+                                                                          img32, (float)Rs, (float)(0.5 * h * h),
+                                                                          phi_out, e_out);
+        };
+        const bool h2 = h > 3e-5 * rho;
+        // blocks of 64 particles from the size where they are two per SM
+        if (total_items >= 304)
+            launch(h2 ? surface_dipole_fp32_kernel<8, 2, true> : surface_dipole_fp32_kernel<8, 2, false>, 64);
+        else
+            launch(h2 ? surface_dipole_fp32_kernel<32, 1, true> : surface_dipole_fp32_kernel<32, 1, false>, 8);
+    } else {
+        surface_pairs_fp32_kernel<<<total_items, kSurfThreads, 0, st>>>(sys, nsys, src_hi, src_lo, ndir, dirs32, img32,
+                                                                       (float)Rs, (float)h, phi_out, e_out);
+    }
+    HSMA_LAUNCHED();
+    HSMA_CUDA_TRY(cudaGetLastError());
+    return HSMA_OK;
+}
+
+__global__ void directions_fp32_kernel(int n, const double4_32a *dirs, float4 *out)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double4_32a u = dirs[i];
+    out[i] = make_float4((float)u.x, (float)u.y, (float)u.z, u.w > 0.0 ? 1.f : 0.f);
+}
+
+int launch_directions_fp32(int n, const double4_32a *dirs, float4 *out, cudaStream_t st)
+{
+    directions_fp32_kernel<<<(n + 255) / 256, 256, 0, st>>>(n, dirs, out);
     HSMA_LAUNCHED();
     HSMA_CUDA_TRY(cudaGetLastError());
     return HSMA_OK;
