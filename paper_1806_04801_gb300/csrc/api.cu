@@ -289,9 +289,12 @@ hsma_tuning choose_tuning(const hsma_plan_s *p, int nsys, const long long *n)
         }
     }
     if (best) return *best;
-    // untuned: the packed variants measured fastest on this part, four targets
-    // per thread for one system, three for a batch
-    return p->precision == HSMA_FP64 ? hsma_tuning{4, 24, 0.0} : hsma_tuning{nsys > 1 ? 17 : 14, 48, 0.0};
+    // untuned FP32: packed variants, two targets per thread where blocks of 384
+    // leave the chip with too few items (step time with 13 / 17 / 14: N = 500
+    // 219 / 224 / 246 us, N = 1000 241 / 257 / 257), three above (N = 4000 451 /
+    // 452 / 486, N = 8000 843 / 815 / 947, N = 16000 2132 / 2117 / 2248)
+    if (p->precision == HSMA_FP64) return hsma_tuning{4, 24, 0.0};
+    return hsma_tuning{batch_work(p, nsys, n) < 1e8 ? 13 : 17, 48, 0.0};
 }
 
 void shape_batch(const hsma_plan_s *p, int nsys, const long long *n, int precision, const hsma_tuning &tu,
