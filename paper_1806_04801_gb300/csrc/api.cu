@@ -504,8 +504,11 @@ int enqueue_update(hsma_plan_s *p, const BatchShape &sh, const Workspace &w, int
 {
     const int nsys = sh.nsys;
     int rc = HSMA_OK;
-    HSMA_CUDA_TRY(cudaMemsetAsync(w.status, 0, sizeof(int) * nsys, st));
-    HSMA_CUDA_TRY(cudaMemsetAsync(w.ctrl, 0, sizeof(int) * 8, st));
+    const bool small = mode != kReuse && sh.max_n <= kSmallSystem;
+    if (!small) {
+        HSMA_CUDA_TRY(cudaMemsetAsync(w.status, 0, sizeof(int) * nsys, st));
+        HSMA_CUDA_TRY(cudaMemsetAsync(w.ctrl, 0, sizeof(int) * 8, st));
+    }
     record(p, st, 0);
     const int *perm = w.perm;
     if (mode == kReuse) {
@@ -548,7 +551,9 @@ int enqueue_update(hsma_plan_s *p, const BatchShape &sh, const Workspace &w, int
     sa.keys2 = w.keys2;
     sa.vals2 = w.vals2;
     sa.hist = w.hist;
-    if ((rc = launch_sort_particles(sa, sh.nblk_max, st))) return rc;
+    if ((rc = small ? launch_sort_small(sa, sh.nblk_max, w.status, w.ctrl, st)
+                    : launch_sort_particles(sa, sh.nblk_max, st)))
+        return rc;
 
     // (a1) in-set
     InsetArgs ia;
@@ -572,7 +577,7 @@ int enqueue_update(hsma_plan_s *p, const BatchShape &sh, const Workspace &w, int
     ia.cen = w.cen;
     ia.cenf = w.cenf;
     ia.qsums = w.qsums;
-    if ((rc = launch_inset(ia, st))) return rc;
+    if ((rc = small ? launch_inset_small(ia, st) : launch_inset(ia, st))) return rc;
     if (mode == kBuild) {
         // candidates within Rs + skin over the enlarged shift table, and the
         // order and positions they refer to

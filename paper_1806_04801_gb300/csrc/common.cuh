@@ -337,6 +337,9 @@ struct SortArgs {
     int *hist;
 };
 int launch_sort_particles(const SortArgs &a, int nblk_max, cudaStream_t st);
+// systems of at most kSmallSystem particles: two launches; also clears
+// status[nsys] and ctrl[8]
+int launch_sort_small(const SortArgs &a, int nblk_max, int *status, int *ctrl, cudaStream_t st);
 int launch_tile_boxes(const SysDesc *sys, int nsys, long long max_tiles, const long long *ns, const float4 *src_hi,
                       int tile, float4 *boxes, cudaStream_t st);
 int launch_gather_targets(int n, const int *perm, const double4_32a *in64, const float4 *inhi, const float4 *inlo,
@@ -366,6 +369,10 @@ struct InsetArgs {
     int2 *cand = nullptr;   // candidate pass only: (spatial index, shift) of each hit
 };
 int launch_inset(const InsetArgs &a, cudaStream_t st);
+// The same for systems of at most kSmallSystem particles each, in three
+// launches (the scatter adds up the counts itself).
+constexpr int kSmallSystem = 4096;
+int launch_inset_small(const InsetArgs &a, cudaStream_t st);
 // The candidate list of a reusable in-set: the same count/scan/scatter over
 // a's shifts and radius (the caller passes the enlarged sphere and shift
 // table, its own counts / ns buffers and a.cand), after launch_inset of the

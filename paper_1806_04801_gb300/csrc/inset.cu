@@ -173,9 +173,27 @@ __global__ void __launch_bounds__(1024) inset_scan_kernel(InsetArgs a)
         atomicOr(&a.status[sys_i], ST_NONNEUTRAL);
 }
 
+// Neutrality of a periodic system of few blocks, by one thread.
+__device__ __forceinline__ void check_neutral(const InsetArgs &a, const SysDesc &sd, int sys_i)
+{
+    if (a.g.bc != HSMA_BC_PERIODIC) return;
+    const double2 *qs = a.qsums + sd.cnt_off / a.n_shifts;
+    double s = 0.0, sa = 0.0;
+    for (int b = 0; b < sd.nblk; ++b) {
+        s += qs[b].x;
+        sa += qs[b].y;
+    }
+    if (fabs(s) > 1e-12 * sa) atomicOr(&a.status[sys_i], ST_NONNEUTRAL);
+}
+
+// SCANNED: a.counts holds the exclusive prefix; otherwise the counts, whose
+// prefix every block adds up for itself (small systems: at most 16 blocks per
+// shift), the last one also the total.
+template <bool SCANNED>
 __global__ void __launch_bounds__(kInsetThreads) inset_scatter_kernel(InsetArgs a)
 {
     __shared__ int wsum[kInsetThreads / 32];
+    __shared__ int psum[kInsetThreads / 32];
     int sys_i = blockIdx.z;
     const SysDesc sd = a.sys[sys_i];
     int blk = blockIdx.x;
@@ -187,19 +205,39 @@ __global__ void __launch_bounds__(kInsetThreads) inset_scatter_kernel(InsetArgs 
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     unsigned m = __ballot_sync(0xffffffffu, hit);
     if (lane == 0) wsum[wid] = __popc(m);
+    const int me = sh * sd.nblk + blk;
+    if (!SCANNED) {
+        int part = 0;
+        for (int i = threadIdx.x; i < me; i += kInsetThreads) part += a.counts[sd.cnt_off + i];
+        part = __reduce_add_sync(0xffffffffu, part);
+        if (lane == 0) psum[wid] = part;
+    }
     __syncthreads();
+    int base = 0, all = 0;
+    if (SCANNED) {
+        base = a.counts[sd.cnt_off + me];
+    } else {
+        for (int w = 0; w < kInsetThreads / 32; ++w) base += psum[w];
+    }
     int before = 0;
-    for (int w = 0; w < wid; ++w) before += wsum[w];
-    before += __popc(m & ((1u << lane) - 1u));
+    for (int w = 0; w < kInsetThreads / 32; ++w) {
+        if (w < wid) before += wsum[w];
+        all += wsum[w];
+    }
+    before += base + __popc(m & ((1u << lane) - 1u));
+    if (!SCANNED && threadIdx.x == 0 && me == a.n_shifts * sd.nblk - 1) {
+        a.ns[sys_i] = base + all;
+        check_neutral(a, sd, sys_i);
+    }
     if (!hit) return;
     if (a.cand) {  // candidate pass: record (spatial index, shift)
-        a.cand[sd.src_off + a.counts[sd.cnt_off + (long long)sh * sd.nblk + blk] + before] = make_int2((int)j, sh);
+        a.cand[sd.src_off + before] = make_int2((int)j, sh);
         return;
     }
     // the image itself in FP64 (positions of the in-set are exact to FP64)
     double x, y, z, q;
     image_of(centred_at(a, sd, j), a.shifts[sh], a.g, x, y, z, q);
-    long long slot = sd.src_off + a.counts[sd.cnt_off + (long long)sh * sd.nblk + blk] + before;
+    const long long slot = sd.src_off + before;
     if (a.src64) a.src64[slot] = make_double4_32a(x, y, z, q);
     if (a.src_hi) {
         float hx, lx, hy, ly, hz, lz;
@@ -364,7 +402,7 @@ int launch_inset_candidates(const InsetArgs &a, cudaStream_t st)
     HSMA_LAUNCHED();
     inset_scan_kernel<<<a.nsys, 1024, 0, st>>>(a);
     HSMA_LAUNCHED();
-    inset_scatter_kernel<<<grid, kInsetThreads, 0, st>>>(a);
+    inset_scatter_kernel<true><<<grid, kInsetThreads, 0, st>>>(a);
     HSMA_LAUNCHED();
     HSMA_CUDA_TRY(cudaGetLastError());
     return HSMA_OK;
@@ -396,7 +434,20 @@ int launch_inset(const InsetArgs &a, cudaStream_t st)
     HSMA_LAUNCHED();
     inset_scan_kernel<<<a.nsys, 1024, 0, st>>>(a);
     HSMA_LAUNCHED();
-    inset_scatter_kernel<<<grid, kInsetThreads, 0, st>>>(a);
+    inset_scatter_kernel<true><<<grid, kInsetThreads, 0, st>>>(a);
+    HSMA_LAUNCHED();
+    HSMA_CUDA_TRY(cudaGetLastError());
+    return HSMA_OK;
+}
+
+int launch_inset_small(const InsetArgs &a, cudaStream_t st)
+{
+    const dim3 grid(a.nblk_max, a.n_shifts, a.nsys);
+    inset_centre_kernel<<<dim3(a.nblk_max, a.nsys), kInsetThreads, 0, st>>>(a);
+    HSMA_LAUNCHED();
+    inset_count_kernel<<<grid, kInsetThreads, 0, st>>>(a);
+    HSMA_LAUNCHED();
+    inset_scatter_kernel<false><<<grid, kInsetThreads, 0, st>>>(a);
     HSMA_LAUNCHED();
     HSMA_CUDA_TRY(cudaGetLastError());
     return HSMA_OK;

@@ -107,6 +107,47 @@ __global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(SortArgs a,
     vout[dst] = val;
 }
 
+// Small systems: the keys sorted by one block per system in one launch where
+// the radix sort takes six.  Key and index make one 24-bit word (at most 16
+// cells per axis and 4096 particles), so any sort gives the stable order: a
+// bitonic sort in shared memory, whose steps of stride <= 32 stay inside a
+// warp's own 64 elements.  Also clears the step's status and counters, which
+// saves two memsets.  (The keys stay a launch of their own, and the centred
+// positions another: their FP64 divisions on one SM took 100 us at N = 4000.)
+constexpr int kSmallThreads = 1024;
+__global__ void __launch_bounds__(kSmallThreads) small_sort_kernel(SortArgs a, int *status, int *ctrl)
+{
+    __shared__ unsigned key[kSmallSystem];
+    const int sys_i = blockIdx.x, tid = threadIdx.x;
+    const SysDesc sd = a.sys[sys_i];
+    const int n = (int)sd.n;
+    if (tid == 0) status[sys_i] = 0;
+    if (sys_i == 0 && tid < 8) ctrl[tid] = 0;
+    int m = 64;
+    while (m < n) m <<= 1;
+    for (int i = tid; i < m; i += kSmallThreads)
+        key[i] = i < n ? ((unsigned)a.keys[sd.part_off + i] << 12) | (unsigned)i : 0xffffffffu;
+    __syncthreads();
+    for (int k = 2; k <= m; k <<= 1)
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            for (int p = tid; p < m / 2; p += kSmallThreads) {
+                const int i = 2 * p - (p & (j - 1)), h = i + j;
+                const unsigned u = key[i], v = key[h];
+                if ((u > v) == ((i & k) == 0)) {
+                    key[i] = v;
+                    key[h] = u;
+                }
+            }
+            // the next step reads other warps' elements only at strides over 32
+            if (j > 32 || (j == 1 && k > 32))
+                __syncthreads();
+            else
+                __syncwarp();
+        }
+    __syncthreads();
+    for (int j = tid; j < n; j += kSmallThreads) a.vals[sd.part_off + j] = (int)(key[j] & 0xfffu);
+}
+
 // Axis-aligned box of every tile of `tile` consecutive in-set entries (high
 // FP32 words), widened by a relative margin that covers the low words.
 __global__ void tile_boxes_kernel(const SysDesc *sys, const long long *ns, const float4 *src_hi, int tile,
@@ -162,6 +203,16 @@ int launch_sort_particles(const SortArgs &a, int nblk_max, cudaStream_t st)
         t = vin; vin = vout; vout = t;
     }
     // after two passes the sorted order is back in keys/vals (a.vals = perm)
+    HSMA_CUDA_TRY(cudaGetLastError());
+    return HSMA_OK;
+}
+
+int launch_sort_small(const SortArgs &a, int nblk_max, int *status, int *ctrl, cudaStream_t st)
+{
+    morton_keys_kernel<<<dim3(nblk_max, a.nsys), kSortThreads, 0, st>>>(a);
+    HSMA_LAUNCHED();
+    small_sort_kernel<<<a.nsys, kSmallThreads, 0, st>>>(a, status, ctrl);
+    HSMA_LAUNCHED();
     HSMA_CUDA_TRY(cudaGetLastError());
     return HSMA_OK;
 }
