@@ -43,6 +43,7 @@ constexpr int kT64 = 1;
 constexpr int kTB64 = kThreads * kT64;
 constexpr int kTile64 = 256;
 constexpr int kFoldFx = 16;             // FxSums::gf fold interval (sources)
+constexpr int kStepFx = 4;              // sources per step
 constexpr int kFold = 32;               // potential fold interval (sources)
 constexpr int kFold2 = 64;              // packed loop: 32 sources per lane
 constexpr bool kCpDouble = true;        // mode 1: two interleaved buffers, one barrier per tile
@@ -526,10 +527,11 @@ __global__ void __launch_bounds__(kThreads, MINB) pair_fp32_kernel(PairArgs a)
 // warps go on (14% busy), so a larger near radius would cost little and a
 // smaller one would cost the field's precision.
 // Bound by the FMA-heavy pipe, which issues the 32 x 32 multiplies (78% of
-// its active cycles; ALU 44%, issue slots 64%); keeping the 64-bit additions
-// apart from the multiplies was 7% slower.  Measured: near-sum phase of
-// N = 9999 (1.96e9 pairs) 61.3 -> 11.1 ms, 3.2e10 -> 1.77e11 pairs/s; N = 1000
-// 1.30 -> 0.24 ms; grounded N = 3001 9.4 -> 1.6 ms.  Error against quad
+// its active cycles with one source per step; ALU 44%, issue slots 64%);
+// keeping the 64-bit additions apart from the multiplies was 7% slower, four
+// sources per step 6% faster than one.  Measured: near-sum phase of N = 9999
+// (1.96e9 pairs) 61.3 -> 10.5 ms, 3.2e10 -> 1.87e11 pairs/s; N = 1000 1.30 ->
+// 0.22 ms; grounded N = 3001 9.4 -> 1.56 ms.  Error against quad
 // precision (N = 300..4000, both boundaries, three charge patterns): field
 // 1.6e-16..8.0e-16 of its norm against 4.7e-16..1.7e-15 before, potential
 // 1.5e-16..3.9e-15 against 3.5e-16..5.2e-15.
@@ -622,7 +624,7 @@ __device__ __noinline__ void tile64(FxShared &sm, int buf, int cnt, const int (&
 }
 
 // A tile in fixed point.  ps, gs: factors of the potential and field sums.
-// Returns how many of the cnt source steps held a near pair in this warp.
+// Returns the most near pairs that a thread of this warp had.
 template <bool FIELD>
 __device__ __forceinline__ int tile_fx(FxShared &sm, int buf, int cnt, const FxTarget (&tg)[kT64],
                                        const int (&self_rel)[kT64], bool skip_zero, double ps, double gs)
@@ -647,43 +649,60 @@ __device__ __forceinline__ int tile_fx(FxShared &sm, int buf, int cnt, const FxT
                 sums[t].gf[c] = 0.f;
             }
     };
+    auto near = [](uint64_t A) { return (uint32_t)(A >> 32) < (uint32_t)(kFxNearA >> 32); };
+    // kStepFx sources per step: one branch for their near pairs, and
+    // independent chains to issue (the slots past cnt hold uncharged sources)
 #pragma unroll 1
-    for (int s = 0; s < cnt; ++s) {
+    for (int s0 = 0; s0 < cnt; s0 += kStepFx) {
         // one FP32 sum over the whole tile would round every term at the
         // closest pairs' magnitude
-        if (FIELD && s % kFoldFx == 0) fold();
-        const FxSource f = sm.fx[s];
-        const int qsign = f.qh >> 31;
-        int dh[kT64][3];
-        uint64_t A[kT64];
+        if (FIELD && s0 % kFoldFx == 0) fold();
+        int dh[kStepFx][kT64][3];
+        uint64_t A[kStepFx][kT64];
         bool any = false;
 #pragma unroll
-        for (int t = 0; t < kT64; ++t) {
-            dh[t][0] = f.hx - tg[t].h[0];
-            dh[t][1] = f.hy - tg[t].h[1];
-            dh[t][2] = f.hz - tg[t].h[2];
-            const int dl[3] = {f.lx - tg[t].l[0], f.ly - tg[t].l[1], f.lz - tg[t].l[2]};
-            A[t] = fx_distance2(dh[t], dl);
-            any = any || A[t] < kFxNearA;
-        }
-        if (any) {
-            ++slow;
-            const double4_32a p = sm.src[buf][s];
+        for (int i = 0; i < kStepFx; ++i) {
+            const FxSource &f = sm.fx[s0 + i];
 #pragma unroll
             for (int t = 0; t < kT64; ++t) {
-                if (A[t] < kFxNearA)
-                    pair64<FIELD>(p, sm.tgt[t][0][tid], sm.tgt[t][1][tid], sm.tgt[t][2][tid], s == self_rel[t],
-                                  skip_zero, sm.acc[t][0][tid], sm.acc[t][1][tid], sm.acc[t][2][tid],
-                                  sm.acc[t][3][tid]);
+                dh[i][t][0] = f.hx - tg[t].h[0];
+                dh[i][t][1] = f.hy - tg[t].h[1];
+                dh[i][t][2] = f.hz - tg[t].h[2];
+                const int dl[3] = {f.lx - tg[t].l[0], f.ly - tg[t].l[1], f.lz - tg[t].l[2]};
+                A[i][t] = fx_distance2(dh[i][t], dl);
+                any = any || near(A[i][t]);
+            }
+        }
+        if (any) {
+#pragma unroll 1
+            for (int i = 0; i < kStepFx && s0 + i < cnt; ++i) {
+                const double4_32a p = sm.src[buf][s0 + i];
+#pragma unroll
+                for (int t = 0; t < kT64; ++t) {
+                    uint64_t Ai = A[0][t];
+#pragma unroll
+                    for (int j = 1; j < kStepFx; ++j) Ai = i == j ? A[j][t] : Ai;
+                    if (near(Ai)) {
+                        ++slow;
+                        pair64<FIELD>(p, sm.tgt[t][0][tid], sm.tgt[t][1][tid], sm.tgt[t][2][tid],
+                                      s0 + i == self_rel[t], skip_zero, sm.acc[t][0][tid], sm.acc[t][1][tid],
+                                      sm.acc[t][2][tid], sm.acc[t][3][tid]);
+                    }
+                }
             }
         }
 #pragma unroll
-        for (int t = 0; t < kT64; ++t) {
-            const FxPair r = fx_inverse(A[t], A[t] < kFxNearA, f.qh, f.ql);
-            fx_add_potential(sums[t], r, f.fq);
-            if (FIELD) {
-                const float df[3] = {f.fx - tg[t].f[0], f.fy - tg[t].f[1], f.fz - tg[t].f[2]};
-                fx_add_field(sums[t], r, dh[t], df, qsign, f.fq);
+        for (int i = 0; i < kStepFx; ++i) {
+            const FxSource &f = sm.fx[s0 + i];
+            const float fq = f.fq;
+#pragma unroll
+            for (int t = 0; t < kT64; ++t) {
+                const FxPair r = fx_inverse(A[i][t], near(A[i][t]), f.qh, f.ql);
+                fx_add_potential(sums[t], r, fq);
+                if (FIELD) {
+                    const float df[3] = {f.fx - tg[t].f[0], f.fy - tg[t].f[1], f.fz - tg[t].f[2]};
+                    fx_add_field(sums[t], r, dh[i][t], df, f.qh >> 31, fq);
+                }
             }
         }
     }
@@ -702,7 +721,7 @@ __device__ __forceinline__ int tile_fx(FxShared &sm, int buf, int cnt, const FxT
     return __reduce_max_sync(0xffffffffu, slow);
 }
 
-__global__ void __launch_bounds__(kThreads, 5) pair_fp64_kernel(PairArgs a)
+__global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem64[];
     FxShared &sm = *reinterpret_cast<FxShared *>(smem64);
@@ -829,6 +848,8 @@ __global__ void __launch_bounds__(kThreads, 5) pair_fp64_kernel(PairArgs a)
             const bool native =
                 blk_native || eq > 1923 || eq < 123 || (qmax != 0u && (int)(qmin >> 20) < eq - 20);
             if (!native) {
+                for (int s = cnt + tid; s < (cnt + kStepFx - 1) / kStepFx * kStepFx; s += kThreads)
+                    sm.fx[s] = FxSource{src_lim, src_lim, src_lim, 0, 0, 0, 0, 0u, 0.f, 0.f, 0.f, 0.f};
                 for (int s = tid; s < cnt; s += kThreads) {
                     fx_split_charge(fx_fixed(sm.src[buf][s].w, 63 + 1022 - eq), sm.fx[s].qh, sm.fx[s].ql,
                                     sm.fx[s].fq);
@@ -845,7 +866,7 @@ __global__ void __launch_bounds__(kThreads, 5) pair_fp64_kernel(PairArgs a)
                 const double ps = rg.scale * exp2i(eq - 1022), fs = ps * rg.scale;
                 const int slow = field ? tile_fx<true>(sm, buf, cnt, tg, self_rel, skip_zero, ps, fs)
                                        : tile_fx<false>(sm, buf, cnt, tg, self_rel, skip_zero, ps, fs);
-                native_tiles = 4 * slow > 3 * cnt ? 7 : 0;
+                native_tiles = 4 * slow > 3 * cnt * kT64 ? 7 : 0;
             }
             __syncthreads();
             if (tid == 0 && k + 2 < ntile) issue(k + 2, buf);

@@ -42,7 +42,7 @@ namespace hsma {
 // y < 7.9 keeps Y below 2^31, and 256 terms |q| / r^2 <= 62.5 below 2^63 in
 // the units of FxSums::g1.
 constexpr double kFxNearR = 1.0 / 7.9;
-constexpr uint64_t kFxNearA = (uint64_t)(kFxNearR * kFxNearR * 1152921504606846976.0);
+constexpr uint64_t kFxNearA = (uint64_t)(kFxNearR * kFxNearR * 1152921504606846976.0) >> 32 << 32;
 
 struct FxSource {
     int hx, hy, hz, qh;
@@ -82,6 +82,10 @@ HSMA_HD void fx_clear(FxSums &s)
         s.gf[c] = 0.f;
     }
 }
+
+// a b / 2^32 to within 2^17: where only its upper half matters, half the cost
+// of the full product on the pipe that bounds the loop.
+HSMA_HD uint32_t fx_mulhi16(uint32_t a, uint32_t b) { return (a >> 16) * (b >> 16); }
 
 HSMA_HD float fx_rsqrt(float x)
 {
@@ -195,7 +199,7 @@ HSMA_HD FxPair fx_inverse(uint64_t A, bool near, int qh, uint32_t ql)
     r.P = (uint64_t)(uint32_t)Y * (uint32_t)Y;
     // (A P - 2^116) / 2^32 in 64 bits, wrapping: -e in units 2^-84
     const uint32_t b0 = (uint32_t)r.P, b1 = (uint32_t)(r.P >> 32);
-    uint64_t acc = (((uint64_t)a0 * b0) >> 32) + (uint64_t)a1 * b0 + (uint64_t)a0 * b1;
+    uint64_t acc = fx_mulhi16(a0, b0) + (uint64_t)a1 * b0 + (uint64_t)a0 * b1;
     acc += (uint64_t)(a1 * b1) << 32;
     const int64_t ne = (int64_t)acc;
     r.ef = -(float)(int)(ne >> 32);
@@ -230,8 +234,8 @@ HSMA_HD void fx_add_field(FxSums &s, const FxPair &r, const int (&dh)[3], const 
     // V = (q0 + x) P / 2^64, rounded: units 2^(64 - 59 - 56) = 2^-51
     const uint64_t Q = (uint64_t)(r.q0 + r.x);
     const uint32_t q0 = (uint32_t)Q, q1 = (uint32_t)(Q >> 32), b0 = (uint32_t)r.P, b1 = (uint32_t)(r.P >> 32);
-    const uint64_t t0 = (uint64_t)q0 * b0, t1 = (uint64_t)q0 * b1, t2 = (uint64_t)q1 * b0;
-    const uint64_t m = (t0 >> 32) + (uint32_t)t1 + (uint32_t)t2 + 0x80000000ull;
+    const uint64_t t1 = (uint64_t)q0 * b1, t2 = (uint64_t)q1 * b0;
+    const uint64_t m = (uint64_t)fx_mulhi16(q0, b0) + (uint32_t)t1 + (uint32_t)t2 + 0x80000000ull;
     const int64_t V = (int64_t)(int)q1 * (int64_t)(int)b1 + (int64_t)(t1 >> 32) + (int64_t)(t2 >> 32) +
                       (int64_t)(m >> 32) - (int64_t)(uint32_t)(qsign & (int)b0);
     const int vh = (int)(V >> 32);
