@@ -1846,17 +1846,8 @@ int hsma_coulomb_sum(int64_t ns, const double *src, int64_t nt, const double *tg
     cudaGetDevice(&dev);
     int sms = 0;
     HSMA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int TB = pair_targets_per_block(precision);
-    const int tile = precision == HSMA_FP64 ? 256 : 512;
-    const int ctas = pair_max_ctas_per_sm(precision);
-    const int slots = sms * ctas;
-    SysDesc d{};
-    d.n = 0;
-    d.ntb_part = 0;
-    d.ntb = (int)((nt + TB - 1) / TB);
-    double chunk = std::max(4.0 * tile, (double)d.ntb * ns / (24.0 * slots));
-    long long maxchunks = std::max(1LL, (long long)((ns + tile - 1) / tile));
-    d.nchunks = (int)std::max(1LL, std::min(maxchunks, (long long)llround(ns / chunk)));
+    const int slots = sms * pair_max_ctas_per_sm(precision, kCoulombVariant);
+    const SysDesc d = coulomb_shape(ns, nt, precision, slots);
     long long items = (long long)d.ntb * d.nchunks;
     if (items > (1LL << 30)) return HSMA_E_ARG;
     const size_t n32 = precision == HSMA_FP64 ? 0 : 1, n64 = 1 - n32;

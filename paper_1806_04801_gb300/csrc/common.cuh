@@ -491,6 +491,8 @@ struct CoulombBuffers {
     double4_32a *s64, *t64;         // FP64 form
     float4 *partials;
 };
+constexpr int kCoulombVariant = 13;  // FP32: two targets per thread, packed (pair.cu)
+SysDesc coulomb_shape(long long ns, long long nt, int precision, int slots);
 int launch_coulomb(const CoulombBuffers &b, const SysDesc &d, long long ns, const double *src, long long nt,
                    const double *tgt, double *pot, double *field, int precision, long long items, int slots,
                    cudaStream_t st);

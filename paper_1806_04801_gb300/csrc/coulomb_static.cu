@@ -194,6 +194,22 @@ int static_setup(int dev, void **addr, int *sms)
 
 }  // namespace
 
+// Targets of a block, chunks of the sources: items of four tiles, of fewer --
+// down to one -- where four would leave less than two items per CTA slot.
+SysDesc coulomb_shape(long long ns, long long nt, int precision, int slots)
+{
+    const int TB = pair_targets_per_block(precision, kCoulombVariant);
+    const double tile = pair_sources_per_tile(precision, kCoulombVariant);
+    SysDesc d{};
+    d.ntb = (int)((nt + TB - 1) / TB);
+    const double work = (double)d.ntb * ns;
+    const double chunk =
+        std::max(std::min(4.0 * tile, std::max(tile, work / (2.0 * slots))), work / (24.0 * slots));
+    const long long most = std::max(1LL, (long long)std::ceil(ns / tile));
+    d.nchunks = (int)std::max(1LL, std::min(most, (long long)llround(ns / chunk)));
+    return d;
+}
+
 // Four launches and no copy: the records are made and the results written by
 // the kernels themselves.
 int launch_coulomb(const CoulombBuffers &b, const SysDesc &d, long long ns, const double *src, long long nt,
@@ -226,7 +242,7 @@ int launch_coulomb(const CoulombBuffers &b, const SysDesc &d, long long ns, cons
     pa.next_item = b.ctrl;
     pa.status = b.status;
     const int grid = (int)std::max(1LL, std::min(items, (long long)slots));
-    int rc = launch_pair(pa, precision, 4, grid, st);
+    int rc = launch_pair(pa, precision, kCoulombVariant, grid, st);
     if (rc) return rc;
     return launch_partial_reduce(b.sys, 1, nt, (int)nt, b.partials, precision, pot, field, st);
 }
@@ -251,16 +267,9 @@ extern "C" int hsma_coulomb_sum_static(int64_t ns, const double *src, int64_t nt
 
     // work decomposition as in hsma_coulomb_sum, with the chunk count lowered
     // until the call fits in the static array
-    const int TB = pair_targets_per_block(precision);
-    const int tile = precision == HSMA_FP64 ? 256 : 512;
-    const int slots = sms * pair_max_ctas_per_sm(precision);
-    SysDesc d{};
-    d.n = 0;
-    d.ntb_part = 0;
-    d.ntb = (int)((nt + TB - 1) / TB);
-    double chunk = std::max(4.0 * tile, (double)d.ntb * ns / (24.0 * slots));
-    long long maxchunks = std::max(1LL, (long long)((ns + tile - 1) / tile));
-    int nchunks = (int)std::max(1LL, std::min(maxchunks, (long long)llround(ns / chunk)));
+    const int slots = sms * pair_max_ctas_per_sm(precision, kCoulombVariant);
+    SysDesc d = coulomb_shape(ns, nt, precision, slots);
+    int nchunks = d.nchunks;
     while (nchunks > 1 && layout_for(ns, nt, nchunks, precision).end > kStaticScratchBytes) nchunks = nchunks / 2;
     StaticLayout L = layout_for(ns, nt, nchunks, precision);
     if (L.end > kStaticScratchBytes) return HSMA_E_CAPACITY;
