@@ -491,9 +491,10 @@ const char *hsma_version(void);
 int64_t hsma_kernel_launches(void);
 
 /* Number of device and pinned-host allocation and free calls (cudaMalloc,
- * cudaFree, cudaMallocHost, cudaFreeHost) this library has made since it was
- * loaded, over all plans and threads: a caller can check with it that a call
- * allocated nothing (no counterpart in the paper). */
+ * cudaFree, their stream-ordered forms, cudaMallocHost, cudaFreeHost) this
+ * library has made since it was loaded, over all plans and threads: a caller
+ * can check with it that a call allocated nothing (no counterpart in the
+ * paper). */
 int64_t hsma_allocation_calls(void);
 
 /* Per-phase device times (milliseconds) of the plan's last update step,

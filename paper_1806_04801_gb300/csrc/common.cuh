@@ -40,6 +40,19 @@ inline cudaError_t dev_free(void *p)
     g_alloc_calls.fetch_add(1, std::memory_order_relaxed);
     return cudaFree(p);
 }
+// Stream-ordered, from the device's default pool (which gives freed memory
+// back at the next synchronisation): for one call's working memory.
+template <class T>
+inline cudaError_t dev_malloc_async(T **p, size_t bytes, cudaStream_t st)
+{
+    g_alloc_calls.fetch_add(1, std::memory_order_relaxed);
+    return cudaMallocAsync(reinterpret_cast<void **>(p), bytes, st);
+}
+inline cudaError_t dev_free_async(void *p, cudaStream_t st)
+{
+    g_alloc_calls.fetch_add(1, std::memory_order_relaxed);
+    return cudaFreeAsync(p, st);
+}
 template <class T>
 inline cudaError_t host_malloc(T **p, size_t bytes)
 {
