@@ -78,6 +78,7 @@ struct Workspace {
     double *phi_out = nullptr, *e_out = nullptr;
     double *energy = nullptr, *upart = nullptr;
     int *status = nullptr;
+    StepResult *result = nullptr;
     int *ctrl = nullptr;                            // work counters
     SysDesc *sys = nullptr;
     float *tc_work = nullptr;
@@ -422,7 +423,8 @@ size_t carve_workspace(const hsma_plan_s *p, const BatchShape &sh, int precision
     w->e_out = c.take<double>(3 * sh.n_total);
     w->energy = c.take<double>(sh.nsys);
     w->upart = c.take<double>((size_t)sh.nsys * finalize_blocks(sh.max_n));
-    w->status = c.take<int>(sh.nsys);
+    w->status = c.take<int>(2 * (size_t)sh.nsys);  // bits, then counters of the last kernel
+    w->result = c.take<StepResult>(sh.nsys);
     w->ctrl = c.take<int>(8);
     w->sys = c.take<SysDesc>(sh.nsys);
     w->tc_work = (precision == HSMA_FP32_TC_FIT) ? (float *)c.take<char>(tc_work_bytes(p->K, p->ncols, sh.nsys, fit_ctas(p)))
@@ -506,7 +508,7 @@ int enqueue_update(hsma_plan_s *p, const BatchShape &sh, const Workspace &w, int
     int rc = HSMA_OK;
     const bool small = mode != kReuse && sh.max_n <= kSmallSystem;
     if (!small) {
-        HSMA_CUDA_TRY(cudaMemsetAsync(w.status, 0, sizeof(int) * nsys, st));
+        HSMA_CUDA_TRY(cudaMemsetAsync(w.status, 0, 2 * sizeof(int) * nsys, st));
         HSMA_CUDA_TRY(cudaMemsetAsync(w.ctrl, 0, sizeof(int) * 8, st));
     }
     record(p, st, 0);
@@ -663,7 +665,7 @@ int enqueue_update(hsma_plan_s *p, const BatchShape &sh, const Workspace &w, int
     }
     if ((rc = launch_finalize(w.sys, nsys, sh.max_n, perm, w.q, w.phi_tgt, w.e_part, w.phi_out, w.e_out,
                               want_f ? w.forces : nullptr, want_p ? w.pot : nullptr, nullptr, w.upart, w.energy,
-                              w.status, st)))
+                              w.ns, w.status, w.result, st)))
         return rc;
     record(p, st, 7);
     return HSMA_OK;
@@ -812,14 +814,11 @@ int run_update(hsma_plan_s *p, int nsys, const int64_t *offsets, const hsma_part
     carve_workspace(p, sh, prec, true, true, p->ws_mem, &w);
     p->ws = w;
     const size_t sys_bytes = align_up(sizeof(SysDesc) * nsys, 64);
-    const size_t pin_bytes = sys_bytes + align_up(sizeof(double) * nsys, 64) + align_up(sizeof(long long) * nsys, 64) +
-                             align_up(sizeof(int) * nsys, 64);
+    const size_t pin_bytes = sys_bytes + align_up(sizeof(StepResult) * nsys, 64);
     rc = ensure_pinned(p, pin_bytes);
     if (rc) return rc;
     SysDesc *hsys = (SysDesc *)p->hpin;
-    double *h_energy = (double *)((char *)p->hpin + sys_bytes);
-    long long *h_ns = (long long *)((char *)h_energy + align_up(sizeof(double) * nsys, 64));
-    int *h_status = (int *)((char *)h_ns + align_up(sizeof(long long) * nsys, 64));
+    StepResult *h_result = (StepResult *)((char *)p->hpin + sys_bytes);
     memcpy(hsys, sh.sys.data(), sizeof(SysDesc) * nsys);
     cudaStream_t st;
     if ((rc = work_stream(p, &st))) return rc;
@@ -840,9 +839,8 @@ int run_update(hsma_plan_s *p, int nsys, const int64_t *offsets, const hsma_part
     auto device_step = [&](int m) -> int {
         int r = launch_step(p, sh, w, prec, want_f, want_p, m, n, st);
         if (r) return r;
-        HSMA_CUDA_TRY(cudaMemcpyAsync(h_energy, w.energy, sizeof(double) * nsys, cudaMemcpyDeviceToHost, st));
-        HSMA_CUDA_TRY(cudaMemcpyAsync(h_status, w.status, sizeof(int) * nsys, cudaMemcpyDeviceToHost, st));
-        HSMA_CUDA_TRY(cudaMemcpyAsync(h_ns, w.ns, sizeof(long long) * nsys, cudaMemcpyDeviceToHost, st));
+        HSMA_CUDA_TRY(
+            cudaMemcpyAsync(h_result, w.result, sizeof(StepResult) * nsys, cudaMemcpyDeviceToHost, st));
         if (m == kBuild)
             HSMA_CUDA_TRY(cudaMemcpyAsync(p->md_ns_host, p->md_ns, sizeof(long long), cudaMemcpyDeviceToHost, st));
         if (want_f) HSMA_CUDA_TRY(cudaMemcpyAsync(forces, w.forces, sizeof(double) * 3 * sh.n_total, out_kind, st));
@@ -852,7 +850,7 @@ int run_update(hsma_plan_s *p, int nsys, const int64_t *offsets, const hsma_part
         return HSMA_OK;
     };
     if ((rc = device_step(mode))) return rc;
-    if (mode == kReuse && (h_status[0] & ST_STALE)) {
+    if (mode == kReuse && (h_result[0].status & ST_STALE)) {
         // a particle moved by the skin or more (or the charges changed): the
         // list no longer covers the in-set; redo the step with a new list
         ++p->md_stale;
@@ -863,7 +861,7 @@ int run_update(hsma_plan_s *p, int nsys, const int64_t *offsets, const hsma_part
     if (mode == kReuse) ++p->md_reuses;
     if (mode == kBuild) {
         ++p->md_builds;
-        p->md_valid = map_status(h_status[0]) == HSMA_OK;
+        p->md_valid = map_status(h_result[0].status) == HSMA_OK;
         p->md_n = n[0];
         p->md_ncand = *p->md_ns_host;
         p->md_prec = prec;
@@ -885,14 +883,14 @@ int run_update(hsma_plan_s *p, int nsys, const int64_t *offsets, const hsma_part
 
     int worst = HSMA_OK;
     for (int s = 0; s < nsys; ++s) {
-        if (energies) energies[s] = h_energy[s];
-        int code = map_status(h_status[s]);
+        if (energies) energies[s] = h_result[s].energy;
+        int code = map_status(h_result[s].status);
         if (status_out) status_out[s] = code;
         if (code != HSMA_OK && worst == HSMA_OK) worst = code;
     }
     if (single) {
-        single->energy = h_energy[0];
-        single->n_inset = h_ns[0];
+        single->energy = h_result[0].energy;
+        single->n_inset = h_result[0].n_inset;
         single->n_images = 6 * (p->F2 + 1);
     }
     return worst;
@@ -1006,7 +1004,7 @@ int run_shard(hsma_plan_s *p, const hsma_particles *x, bool far_stage, int part,
     HSMA_CUDA_TRY(cudaMemcpyAsync(w.sys, p->hpin, sizeof(SysDesc), cudaMemcpyHostToDevice, st));
     HSMA_CUDA_TRY(cudaMemcpyAsync(w.xyz, x->xyz, sizeof(double) * 3 * n, in_kind, st));
     HSMA_CUDA_TRY(cudaMemcpyAsync(w.q, x->q, sizeof(double) * n, in_kind, st));
-    HSMA_CUDA_TRY(cudaMemsetAsync(w.status, 0, sizeof(int), st));
+    HSMA_CUDA_TRY(cudaMemsetAsync(w.status, 0, 2 * sizeof(int), st));
     HSMA_CUDA_TRY(cudaMemsetAsync(w.ctrl, 0, sizeof(int) * 8, st));
 
     // sort and in-set (both stages: the far stage needs the particles in
@@ -1114,7 +1112,8 @@ int run_shard(hsma_plan_s *p, const hsma_particles *x, bool far_stage, int part,
                                           cudaMemcpyHostToDevice, st));
         }
         if ((rc = launch_finalize(w.sys, 1, std::max<long long>(cnt, 1), w.perm, w.q, w.phi_tgt, w.e_part,
-                                  w.phi_out, w.e_out, w.forces, w.pot, w.idx64, w.upart, w.energy, w.status, st)))
+                                  w.phi_out, w.e_out, w.forces, w.pot, w.idx64, w.upart, w.energy, w.ns, w.status,
+                                  w.result, st)))
             return rc;
     }
     std::vector<long long> idx(std::max<long long>(cnt, 1));

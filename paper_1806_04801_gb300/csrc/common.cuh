@@ -351,7 +351,7 @@ struct SortArgs {
 };
 int launch_sort_particles(const SortArgs &a, int nblk_max, cudaStream_t st);
 // systems of at most kSmallSystem particles: two launches; also clears
-// status[nsys] and ctrl[8]
+// status[2 nsys] and ctrl[8]
 int launch_sort_small(const SortArgs &a, int nblk_max, int *status, int *ctrl, cudaStream_t st);
 int launch_tile_boxes(const SysDesc *sys, int nsys, long long max_tiles, const long long *ns, const float4 *src_hi,
                       int tile, float4 *boxes, cudaStream_t st);
@@ -488,11 +488,18 @@ int launch_surface_pairs(const SysDesc *sys, int nsys, int total_items, const fl
 int launch_series_field(const SysDesc *sys, int nsys, long long max_n, int P, double Rs, const double *norm,
                         const double *A, const float4 *src_hi, const float4 *src_lo, const double4_32a *src64,
                         double *phi_out, double *e_out, cudaStream_t st);
+// What the host reads of a system after a step.
+struct StepResult {
+    double energy;
+    long long n_inset;
+    int status, pad;
+};
 int finalize_blocks(long long max_n);
+// status: [nsys] bits, then [nsys] counters, zero at the start of the step
 int launch_finalize(const SysDesc *sys, int nsys, long long max_n, const int *perm, const double *q,
                     const double *phi_tgt, const double *e_part, const double *phi_out, const double *e_out,
-                    double *forces, double *pot, long long *owned_idx, double *upart, double *energy, int *status,
-                    cudaStream_t st);
+                    double *forces, double *pot, long long *owned_idx, double *upart, double *energy,
+                    const long long *ns, int *status, StepResult *result, cudaStream_t st);
 
 // coulomb_static.cu: the direct sum of one call on the caller's buffers.
 struct CoulombBuffers {

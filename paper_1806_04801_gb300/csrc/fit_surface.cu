@@ -623,15 +623,24 @@ __global__ void __launch_bounds__(128) surface_dipole_fp64_kernel(
 constexpr int kFinalThreads = 256;
 constexpr int kFinal = 256;  // one particle per thread: 2048 left one or two blocks to systems of a few thousand
 
+// The block that finishes last in its system (status[nsys + s] counts them)
+// adds the partials -- a warp, each lane every 32nd in order, then a fixed
+// tree, so the sum does not depend on which block it is -- and packs what the
+// host reads into one record.
 __global__ void __launch_bounds__(kFinalThreads) finalize_kernel(const SysDesc *sys, const int *perm, const double *q,
                                                                  const double *phi_tgt, const double *e_part,
                                                                  const double *phi_out, const double *e_out,
                                                                  double *forces, double *pot, long long *owned_idx,
-                                                                 double *upart, int nb_max, int *status)
+                                                                 double *upart, int nb_max, double *energy,
+                                                                 const long long *ns, int *status,
+                                                                 StepResult *result)
 {
     __shared__ double red[32];
+    __shared__ int s_last;
     const int s = blockIdx.y;
     const SysDesc sd = sys[s];
+    const int nb = max(1, (int)((sd.sp_n + kFinal - 1) / kFinal));
+    if ((int)blockIdx.x >= nb) return;
     const long long i0 = sd.sp_lo + (long long)blockIdx.x * kFinal;
     const long long i1 = sd.sp_lo + sd.sp_n;
     double u = 0.0;
@@ -660,22 +669,22 @@ __global__ void __launch_bounds__(kFinalThreads) finalize_kernel(const SysDesc *
     }
     if (bad) atomicOr(&status[s], ST_COINCIDENT);
     u = block_sum(u, red);
-    if (threadIdx.x == 0) upart[(long long)s * nb_max + blockIdx.x] = u;
-}
-
-// U = 1/2 sum of the block partials (of the owned range): a warp, each lane
-// every 32nd partial in order, then a fixed tree.
-__global__ void energy_kernel(const SysDesc *sys, const double *upart, int nb_max, double *energy, int *status)
-{
-    const int s = blockIdx.x;
-    const SysDesc sd = sys[s];
-    const int nb = (int)((sd.sp_n + kFinal - 1) / kFinal);
-    double u = 0.0;
-    for (int b = threadIdx.x; b < nb; b += 32) u += upart[(long long)s * nb_max + b];
+    double *up = upart + (long long)s * nb_max;
+    if (threadIdx.x == 0) {
+        up[blockIdx.x] = u;
+        __threadfence();
+        s_last = atomicAdd(&status[gridDim.y + s], 1) == nb - 1;
+    }
+    __syncthreads();
+    if (!s_last || threadIdx.x >= 32) return;
+    __threadfence();
+    u = 0.0;
+    for (int b = threadIdx.x; b < nb; b += 32) u += __ldcg(up + b);
     u = warp_sum(u);
     if (threadIdx.x != 0) return;
     energy[s] = 0.5 * u;
-    if (!isfinite(u)) atomicOr(&status[s], ST_COINCIDENT);
+    const int st = atomicOr(&status[s], isfinite(u) ? 0 : ST_COINCIDENT) | (isfinite(u) ? 0 : ST_COINCIDENT);
+    result[s] = StepResult{0.5 * u, ns[s], st, 0};
 }
 
 }  // namespace
@@ -760,14 +769,13 @@ int finalize_blocks(long long max_n) { return (int)((max_n + kFinal - 1) / kFina
 
 int launch_finalize(const SysDesc *sys, int nsys, long long max_n, const int *perm, const double *q,
                     const double *phi_tgt, const double *e_part, const double *phi_out, const double *e_out,
-                    double *forces, double *pot, long long *owned_idx, double *upart, double *energy, int *status,
-                    cudaStream_t st)
+                    double *forces, double *pot, long long *owned_idx, double *upart, double *energy,
+                    const long long *ns, int *status, StepResult *result, cudaStream_t st)
 {
     const int nb_max = finalize_blocks(max_n);
     finalize_kernel<<<dim3(nb_max, nsys), kFinalThreads, 0, st>>>(sys, perm, q, phi_tgt, e_part, phi_out, e_out,
-                                                                  forces, pot, owned_idx, upart, nb_max, status);
-    HSMA_LAUNCHED();
-    energy_kernel<<<nsys, 32, 0, st>>>(sys, upart, nb_max, energy, status);
+                                                                  forces, pot, owned_idx, upart, nb_max, energy, ns,
+                                                                  status, result);
     HSMA_LAUNCHED();
     HSMA_CUDA_TRY(cudaGetLastError());
     return HSMA_OK;

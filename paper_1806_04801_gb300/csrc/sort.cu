@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(kSmallThreads) small_sort_kernel(SortArgs a, i
     const int sys_i = blockIdx.x, tid = threadIdx.x;
     const SysDesc sd = a.sys[sys_i];
     const int n = (int)sd.n;
-    if (tid == 0) status[sys_i] = 0;
+    if (tid == 0) status[sys_i] = status[gridDim.x + sys_i] = 0;
     if (sys_i == 0 && tid < 8) ctrl[tid] = 0;
     int m = 64;
     while (m < n) m <<= 1;
