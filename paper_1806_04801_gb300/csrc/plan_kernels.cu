@@ -120,7 +120,9 @@ __global__ void quadrature_kernel(int F2, int F1, double Rs, double4_32a *dirs)
 // left one block per SM).  Four FP64 operations per recurrence step and one
 // per stored value; FP64 issue is slow on this part.
 constexpr int kBasisMaxP = 40;
-constexpr int kBasisWarps = 2;  // warps per block
+// Warps per block: two, or as many as basis_warps finds (the kernels are built
+// for both limits: code built for 12 warps was 7% slower with the same number).
+constexpr int kBasisWarps = 12;
 static_assert(kBasisMaxP == kBasisTableMaxP, "one coefficient table serves both basis forms");
 
 // The recurrence coefficients of every n, m <= kBasisMaxP in FP64, computed
@@ -161,7 +163,8 @@ __host__ __device__ constexpr size_t basis_smem_bytes(int P, int warps)
                 (size_t)warps * 32 * ((size_t)4 * (P + 1) + (size_t)(2 * P + 1)));
 }
 
-__global__ void __launch_bounds__(32 * kBasisWarps) basis_kernel(const __grid_constant__ BasisF64Tables tabs, int P,
+template <int kWarps>
+__global__ void __launch_bounds__(32 * kWarps) basis_kernel(const __grid_constant__ BasisF64Tables tabs, int P,
                                                                  double inv_rs, long long np,
                                                                  const double *__restrict__ pts, int stride,
                                                                  double *__restrict__ out, int ld)
@@ -361,7 +364,6 @@ __device__ __forceinline__ double df_to_f64_scaled(float2 v, uint32_t kb, int k)
 // The recurrence coefficients do not depend on P: the host computes them once
 // in FP64 for every n, m <= 40, splits them into pairs and passes them as a
 // kernel parameter; each block copies the (P+1)^2 it needs to shared memory.
-constexpr int kBasisDfWarps = 2;  // warps per block
 
 __host__ __device__ constexpr size_t basis_df_smem_bytes(int P, int warps)
 {
@@ -458,7 +460,8 @@ __device__ __forceinline__ void basis_df_rows(int P, const float2 *ta, const flo
     }
 }
 
-__global__ void __launch_bounds__(32 * kBasisDfWarps) basis_df_kernel(const __grid_constant__ BasisDfTables tabs,
+template <int kWarps>
+__global__ void __launch_bounds__(32 * kWarps) basis_df_kernel(const __grid_constant__ BasisDfTables tabs,
                                                                       int P, double inv_rs, long long np,
                                                                       const double *__restrict__ pts, int stride,
                                                                       double *__restrict__ out, long long ld)
@@ -711,6 +714,33 @@ int launch_quadrature(int F2, int F1, double Rs, double4_32a *dirs, cudaStream_t
     return HSMA_OK;
 }
 
+// Warps per block.  Blocks of two copy the tables often and leave shared
+// memory unused (10 warps per SM at p = 12, 2 from p = 29 on); a larger block
+// is taken where it brings a tenth more warps.  Not 5, 9 or 10 per SM: one or
+// two of its four sub-partitions then have a warp more than the others, which
+// all wait for (p = 25 in double float 829 us with five against 745 with four,
+// p = 14 411 with ten against 395 with eight).  Both forms take the same shared
+// memory; a block has 1 KB of its own.  Measured, in double float: 1e6 points
+// at p = 12 601 -> 544 us, 3e5 at p = 20 543 -> 491, 2e5 at p = 22 523 -> 450,
+// 6e4 at p = 32 619 -> 403; FP64: p = 20 956 -> 870, p = 22 1018 -> 752.
+static int basis_warps(int P, long long groups, int sms)
+{
+    auto per_sm = [&](int w) {
+        return w * (int)std::min<size_t>({228 * 1024 / (basis_smem_bytes(P, w) + 1024), (size_t)(64 / w), (size_t)32});
+    };
+    int best = 2, most = per_sm(2);
+    const int two = most;
+    for (int w = 1; w <= kBasisWarps; ++w) {
+        if (w > 2 && groups < (long long)w * sms) break;
+        const int n = per_sm(w);
+        if (n > most && 10 * n >= 11 * two && n != 5 && n != 9 && n != 10) {
+            most = n;
+            best = w;
+        }
+    }
+    return best;
+}
+
 int launch_basis(int P, double Rs, long long np, const double *pts, int stride, double *out, long long ld,
                  cudaStream_t st)
 {
@@ -720,14 +750,15 @@ int launch_basis(int P, double Rs, long long np, const double *pts, int stride, 
     int dev = 0, sms = 1, per_sm = 0;
     HSMA_CUDA_TRY(cudaGetDevice(&dev));
     HSMA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const size_t smem = basis_smem_bytes(P, kBasisWarps);
-    HSMA_CUDA_TRY(cudaFuncSetAttribute(basis_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    HSMA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, basis_kernel, 32 * kBasisWarps, smem));
-    if (per_sm < 1) return HSMA_E_ARG;
     const long long groups = (np + 31) / 32;
-    const long long blocks = std::min<long long>((groups + kBasisWarps - 1) / kBasisWarps, (long long)sms * per_sm);
-    basis_kernel<<<(unsigned)blocks, 32 * kBasisWarps, smem, st>>>(basis_f64_tables(), P, 1.0 / Rs, np, pts, stride,
-                                                                   out, (int)ld);
+    const int warps = basis_warps(P, groups, sms);
+    const size_t smem = basis_smem_bytes(P, warps);
+    auto kernel = warps <= 2 ? basis_kernel<2> : basis_kernel<kBasisWarps>;
+    HSMA_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    HSMA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32 * warps, smem));
+    if (per_sm < 1) return HSMA_E_ARG;
+    const long long blocks = std::min<long long>((groups + warps - 1) / warps, (long long)sms * per_sm);
+    kernel<<<(unsigned)blocks, 32 * warps, smem, st>>>(basis_f64_tables(), P, 1.0 / Rs, np, pts, stride, out, (int)ld);
     HSMA_LAUNCHED();
     HSMA_CUDA_TRY(cudaGetLastError());
     return HSMA_OK;
@@ -742,15 +773,15 @@ int launch_basis_df(int P, double Rs, long long np, const double *pts, int strid
     int dev = 0, sms = 1, per_sm = 0;
     HSMA_CUDA_TRY(cudaGetDevice(&dev));
     HSMA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const size_t smem = basis_df_smem_bytes(P, kBasisDfWarps);
-    HSMA_CUDA_TRY(cudaFuncSetAttribute(basis_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    HSMA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, basis_df_kernel, 32 * kBasisDfWarps, smem));
-    if (per_sm < 1) return HSMA_E_ARG;
     const long long groups = (np + 31) / 32;
-    const long long blocks =
-        std::min<long long>((groups + kBasisDfWarps - 1) / kBasisDfWarps, (long long)sms * per_sm);
-    basis_df_kernel<<<(unsigned)blocks, 32 * kBasisDfWarps, smem, st>>>(basis_df_tables(), P, 1.0 / Rs, np, pts,
-                                                                       stride, out, ld);
+    const int warps = basis_warps(P, groups, sms);
+    const size_t smem = basis_df_smem_bytes(P, warps);
+    auto kernel = warps <= 2 ? basis_df_kernel<2> : basis_df_kernel<kBasisWarps>;
+    HSMA_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    HSMA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32 * warps, smem));
+    if (per_sm < 1) return HSMA_E_ARG;
+    const long long blocks = std::min<long long>((groups + warps - 1) / warps, (long long)sms * per_sm);
+    kernel<<<(unsigned)blocks, 32 * warps, smem, st>>>(basis_df_tables(), P, 1.0 / Rs, np, pts, stride, out, ld);
     HSMA_LAUNCHED();
     HSMA_CUDA_TRY(cudaGetLastError());
     return HSMA_OK;
