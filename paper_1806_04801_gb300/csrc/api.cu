@@ -324,11 +324,13 @@ void shape_batch(const hsma_plan_s *p, int nsys, const long long *n, int precisi
         (double)std::max(1, tu.items_per_slot) * slots * (p->preemptible ? kPreemptibleItemsFactor : 1);
     // smallest chunk: four tiles (each item re-reads its targets and writes a
     // partial record per target, which the chunk reduction reads back), less --
-    // down to one tile -- where four would give fewer than two items per CTA
-    // slot (small systems; measured at N = 1000 / 2000: 0.293 -> 0.242 and
-    // 0.315 -> 0.290 ms per step, N >= 1e4 unchanged)
+    // down to one tile -- where four would give fewer than eight items per CTA
+    // slot: with two, the last items left part of the chip idle (step time with
+    // two -> eight: FP64 N = 1000 562 -> 527 us, N = 2000 1174 -> 1079, grounded
+    // N = 3001 1970 -> 1900; FP32 variant 17 N = 4000 392 -> 379, N = 8000 775 ->
+    // 757; sixteen is slower from N = 8000 on, FP32 N >= 16000 alike)
     const double chunk =
-        std::max(std::min(4.0 * tile, std::max(1.0 * tile, work / (2.0 * slots))), work / items_wanted);
+        std::max(std::min(4.0 * tile, std::max(1.0 * tile, work / (8.0 * slots))), work / items_wanted);
     long long part = 0, src = 0, tgt = 0, rec = 0, cnt = 0, hist = 0, tiles = 0, max_tiles = 0;
     long long items = 0, surf = 0;
     int nblk_max = 1;
