@@ -67,6 +67,21 @@ inline cudaError_t host_free(void *p)
 
 void set_last_cuda_error(cudaError_t e, const char *what, const char *file, int line);
 
+// Kernels loaded now.  The runtime loads a kernel at its first use, and that
+// load can wait for the work already on the device, while every other load
+// waits behind it: concurrent lanes load what they may launch before they start.
+template <class... K>
+int load_kernels(K... kernel)
+{
+    cudaFuncAttributes a;
+    for (cudaError_t e : {cudaFuncGetAttributes(&a, kernel)...}) HSMA_CUDA_TRY(e);
+    return HSMA_OK;
+}
+int load_sort_kernels();
+int load_inset_kernels();
+int load_pair_kernels();
+int load_surface_kernels();
+
 // Device status bits, one int per system; the host maps them to codes.
 enum : int {
     ST_NONNEUTRAL = 1,

@@ -781,6 +781,14 @@ int launch_finalize(const SysDesc *sys, int nsys, long long max_n, const int *pe
     return HSMA_OK;
 }
 
+int load_surface_kernels()
+{
+    return load_kernels(fit_fp64_kernel<8>, fit_fp64_kernel<1>, surface_charges_kernel, surface_pairs_fp32_kernel,
+                        surface_pairs_fp64_kernel, surface_dipole_fp64_kernel, surface_dipole_fp32_kernel<8, 2, true>,
+                        surface_dipole_fp32_kernel<8, 2, false>, surface_dipole_fp32_kernel<32, 1, true>,
+                        surface_dipole_fp32_kernel<32, 1, false>, finalize_kernel);
+}
+
 }  // namespace hsma
 
 namespace hsma {

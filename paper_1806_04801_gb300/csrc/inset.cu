@@ -453,4 +453,10 @@ int launch_inset_small(const InsetArgs &a, cudaStream_t st)
     return HSMA_OK;
 }
 
+int load_inset_kernels()
+{
+    return load_kernels(inset_centre_kernel, inset_count_kernel, inset_scan_kernel, inset_scatter_kernel<true>,
+                        inset_scatter_kernel<false>);
+}
+
 }  // namespace hsma

@@ -1116,4 +1116,12 @@ int launch_partial_reduce(const SysDesc *sys, int nsys, long long max_tgt, int n
     return HSMA_OK;
 }
 
+int load_pair_kernels()
+{
+    return load_kernels(pair_fp64_kernel, pair_fp32_kernel<2, 6, 0>, pair_fp32_kernel<4, 5, 0>,
+                        pair_fp32_kernel<4, 4, 0>, pair_fp32_kernel<2, 6, 1>, pair_fp32_kernel<2, 5, 1>,
+                        pair_fp32_kernel<4, 3, 1>, pair_fp32_kernel<4, 4, 2>, pair_fp32_kernel<2, 6, 2>,
+                        pair_fp32_kernel<3, 4, 1>, partial_reduce_kernel<true>, partial_reduce_kernel<false>);
+}
+
 }  // namespace hsma

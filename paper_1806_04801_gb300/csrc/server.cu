@@ -287,7 +287,20 @@ int hsma_server_create(hsma_server_t *out, const double box[3], int bc, int p, d
     // One- and two-system steps of a few charges on every lane before serving:
     // the CUDA runtime loads a kernel at its first launch, and a load can wait
     // for the work already on the device -- a lane's first request would
-    // otherwise queue behind a large batch on another lane.
+    // otherwise queue behind a large batch on another lane.  The kernels that
+    // only larger systems take are loaded without a launch (left to their first
+    // one, a load behind a 2e5-charge batch held up every lane: 206 and 194 ms
+    // for a 4e4- and a 2000-charge request in a fresh process).
+    {
+        int rc = hsma::load_sort_kernels();
+        if (!rc) rc = hsma::load_inset_kernels();
+        if (!rc) rc = hsma::load_pair_kernels();
+        if (!rc) rc = hsma::load_surface_kernels();
+        if (rc) {
+            hsma_server_destroy(s);
+            return rc;
+        }
+    }
     {
         const int nw = 8;
         std::vector<double> wx(3 * 2 * nw), wq(2 * nw), we(2), wf(3 * 2 * nw);

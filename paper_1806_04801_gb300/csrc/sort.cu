@@ -207,6 +207,12 @@ int launch_sort_particles(const SortArgs &a, int nblk_max, cudaStream_t st)
     return HSMA_OK;
 }
 
+int load_sort_kernels()
+{
+    return load_kernels(morton_keys_kernel, radix_hist_kernel, radix_scan_kernel, radix_scatter_kernel,
+                        small_sort_kernel, tile_boxes_kernel);
+}
+
 int launch_sort_small(const SortArgs &a, int nblk_max, int *status, int *ctrl, cudaStream_t st)
 {
     morton_keys_kernel<<<dim3(nblk_max, a.nsys), kSortThreads, 0, st>>>(a);
