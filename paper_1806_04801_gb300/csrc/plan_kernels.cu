@@ -118,11 +118,14 @@ __global__ void quadrature_kernel(int F2, int F1, double Rs, double4_32a *dirs)
 // of one thread per row kept every row's sectors partly written until the
 // row was done: L2 evicted and re-read them, and capping the rows in flight
 // left one block per SM).  Four FP64 operations per recurrence step and one
-// per stored value; FP64 issue is slow on this part.
+// per stored value; FP64 issue is slow on this part.  S warps share a group of
+// points: warp w takes the orders w, w + S, ..., whose recurrences need no
+// other, warp 0 the powers as well, one degree ahead, and all of them store
+// the degree's segments, between two barriers of the group's own warps.
 constexpr int kBasisMaxP = 40;
-// Warps per block: two, or as many as basis_warps finds (the kernels are built
-// for both limits: code built for 12 warps was 7% slower with the same number).
-constexpr int kBasisWarps = 12;
+// Groups of one warp per block: two, or as many as basis_shape finds (the
+// kernels are built for both limits: code built for 12 was 7% slower with two).
+constexpr int kBasisGroups = 12;
 static_assert(kBasisMaxP == kBasisTableMaxP, "one coefficient table serves both basis forms");
 
 // The recurrence coefficients of every n, m <= kBasisMaxP in FP64, computed
@@ -155,19 +158,29 @@ const BasisF64Tables &basis_f64_tables()
     return t;
 }
 
-__host__ __device__ constexpr size_t basis_smem_bytes(int P, int warps)
+__host__ __device__ constexpr size_t basis_smem_bytes(int P, int groups)
 {
-    // tables a, b ((P+1)^2 each), D, E (P+1 each); per warp: 4 (P+1) state
+    // tables a, b ((P+1)^2 each), D, E (P+1 each); per group: 4 (P+1) state
     // slots x 32 lanes and a 32 x (2P+1) staging tile (8-byte words)
     return 8 * ((size_t)2 * (P + 1) * (P + 1) + (size_t)2 * (P + 1) +
-                (size_t)warps * 32 * ((size_t)4 * (P + 1) + (size_t)(2 * P + 1)));
+                (size_t)groups * 32 * ((size_t)4 * (P + 1) + (size_t)(2 * P + 1)));
 }
 
-template <int kWarps>
-__global__ void __launch_bounds__(32 * kWarps) basis_kernel(const __grid_constant__ BasisF64Tables tabs, int P,
-                                                                 double inv_rs, long long np,
-                                                                 const double *__restrict__ pts, int stride,
-                                                                 double *__restrict__ out, int ld)
+// Barrier of the S warps of one group of points (sub: its place in the block).
+template <int S>
+__device__ __forceinline__ void group_sync(int sub)
+{
+    if constexpr (S == 1)
+        __syncwarp();
+    else
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + sub), "n"(32 * S) : "memory");
+}
+
+template <int S, int kThreads>
+__global__ void __launch_bounds__(kThreads) basis_kernel(const __grid_constant__ BasisF64Tables tabs, int P,
+                                                         double inv_rs, long long np,
+                                                         const double *__restrict__ pts, int stride,
+                                                         double *__restrict__ out, int ld)
 {
     extern __shared__ double bsm[];
     const int W = P + 1, pitch = 2 * P + 1;
@@ -181,84 +194,101 @@ __global__ void __launch_bounds__(32 * kWarps) basis_kernel(const __grid_constan
         te[m] = tabs.e[m];
     }
     __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double *wb = te + W + (size_t)warp * 32 * (4 * W + pitch);
+    const int sub = threadIdx.x / (32 * S), w = (threadIdx.x >> 5) % S, lane = threadIdx.x & 31;
+    const int per_block = blockDim.x / (32 * S);
+    double *wb = te + W + (size_t)sub * 32 * (4 * W + pitch);
     double *pst = wb + lane;  // Pbar at even, then odd degrees; slot m at [32 m]
     double *cs = wb + 64 * W + lane, *ss = wb + 96 * W + lane;
     double *stage = wb + 128 * W;  // [32 rows][pitch]
     const long long ngroups = (np + 31) / 32;
-    for (long long g = (long long)blockIdx.x * (blockDim.x >> 5) + warp; g < ngroups;
-         g += (long long)gridDim.x * (blockDim.x >> 5)) {
+    for (long long g = (long long)blockIdx.x * per_block + sub; g < ngroups; g += (long long)gridDim.x * per_block) {
         const long long i0 = g * 32;
         const int rows = (int)min(32LL, np - i0);
         const long long i = i0 + min(lane, rows - 1);  // lanes past the end repeat the last point, unwritten
         const double x = pts[i * stride] * inv_rs, y = pts[i * stride + 1] * inv_rs, z = pts[i * stride + 2] * inv_rs;
         const double r2 = x * x + y * y + z * z;
-        double C = 1.0, S = 0.0;  // (x + i y)^n
+        double C = 1.0, T = 0.0;  // (x + i y)^n
         double *sc0 = stage + lane * pitch;
         double *og = out + i0 * ld;
         for (int n = 0; n <= P; ++n) {
             double *cur = pst + (n & 1) * 32 * W, *prv = pst + ((n & 1) ^ 1) * 32 * W;
             double *sc = sc0 + n;  // column n + m holds the cosine part, n - m the sine part
-            if (n > 0) {
-                const double c2 = C * x - S * y;
-                S = S * x + C * y;
-                C = c2;
-            }
-            cs[32 * n] = C;
-            ss[32 * n] = S;
-            cur[32 * n] = td[n];  // m = n
-            sc[n] = td[n] * C;
-            if (n > 0) {
-                sc[-n] = td[n] * S;
-                const int m = n - 1;  // m = n - 1
-                const double p = te[m] * z;
-                cur[32 * m] = p;
-                sc[m] = p * cs[32 * m];
-                if (m > 0) sc[-m] = p * ss[32 * m];
-            }
             const double *an = ta + n, *bn = tb + n;
-            if (n >= 2) {  // m = 0: (x + i y)^0 = 1
-                const double pn = fma(an[0] * z, prv[0], -(bn[0] * r2) * cur[0]);
+            if constexpr (S == 1) {
+                if (n > 0) {
+                    const double c2 = C * x - T * y;
+                    T = T * x + C * y;
+                    C = c2;
+                }
+                cs[32 * n] = C;
+                ss[32 * n] = T;
+                cur[32 * n] = td[n];  // m = n
+                sc[n] = td[n] * C;
+                if (n > 0) {
+                    sc[-n] = td[n] * T;
+                    const int m = n - 1;  // m = n - 1
+                    const double p = te[m] * z;
+                    cur[32 * m] = p;
+                    sc[m] = p * cs[32 * m];
+                    if (m > 0) sc[-m] = p * ss[32 * m];
+                }
+            } else if (w == 0 && n < P) {  // the next power: its warp reads it after this degree's barriers
+                const double c2 = C * x - T * y;
+                T = T * x + C * y;
+                C = c2;
+                cs[32 * (n + 1)] = C;
+                ss[32 * (n + 1)] = T;
+            }
+            if (w == 0 && (S > 1 || n >= 2)) {  // m = 0: (x + i y)^0 = 1
+                const double pn = n >= 2   ? fma(an[0] * z, prv[0], -(bn[0] * r2) * cur[0])
+                                  : n == 1 ? te[0] * z
+                                           : td[0];
                 cur[0] = pn;
                 sc[0] = pn;
             }
             // m >= 1, four orders per pass: all loads before the stores, which
             // the compiler cannot reorder, so that one warp per sub-partition
-            // (p = 25) keeps the FP64 pipe busier (2.5e5 points 1499 -> 1367
-            // us; 1e6 at p = 12 1028 -> 996)
-            int m = 1;
-            for (; m + 5 <= n; m += 4) {
+            // keeps the FP64 pipe busier
+            int m = w == 0 ? S : w;
+            for (; m + 3 * S + 2 <= n; m += 4 * S) {
                 double p[4], c[4], t[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    p[i] = fma(an[(m + i) * W] * z, prv[32 * (m + i)], -(bn[(m + i) * W] * r2) * cur[32 * (m + i)]);
-                    c[i] = cs[32 * (m + i)];
-                    t[i] = ss[32 * (m + i)];
+                    const int k = m + i * S;
+                    p[i] = fma(an[k * W] * z, prv[32 * k], -(bn[k * W] * r2) * cur[32 * k]);
+                    c[i] = cs[32 * k];
+                    t[i] = ss[32 * k];
                 }
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    cur[32 * (m + i)] = p[i];
-                    sc[m + i] = p[i] * c[i];
-                    sc[-m - i] = p[i] * t[i];
+                    const int k = m + i * S;
+                    cur[32 * k] = p[i];
+                    sc[k] = p[i] * c[i];
+                    sc[-k] = p[i] * t[i];
                 }
             }
-            for (; m + 2 <= n; ++m) {
+            for (; m + 2 <= n; m += S) {
                 const double pn = fma(an[m * W] * z, prv[32 * m], -(bn[m * W] * r2) * cur[32 * m]);
                 cur[32 * m] = pn;
                 sc[m] = pn * cs[32 * m];
                 sc[-m] = pn * ss[32 * m];
             }
-            __syncwarp();
+            if (S > 1 && m <= n) {  // m = n or n - 1
+                const double pn = m == n ? td[m] : te[m] * z;
+                cur[32 * m] = pn;
+                sc[m] = pn * cs[32 * m];
+                sc[-m] = pn * ss[32 * m];
+            }
+            group_sync<S>(sub);
             const int wd = 2 * n + 1, tot = rows * wd;
             const uint32_t cw = ((1u << 20) + (uint32_t)wd - 1u) / (uint32_t)wd;  // ceil(2^20 / (2n + 1))
             double *ob = og + n * n;
 #pragma unroll 4
-            for (int f = lane; f < tot; f += 32) {
+            for (int f = lane + 32 * w; f < tot; f += 32 * S) {
                 const int r = (int)(((uint32_t)f * cw) >> 20), j = f - r * wd;
                 ob[r * ld + j] = stage[r * pitch + j];
             }
-            __syncwarp();
+            group_sync<S>(sub);
         }
     }
 }
@@ -390,12 +420,12 @@ __device__ __forceinline__ double df_to_f64_scaled(float2 v, uint32_t kb, int k)
 // in FP64 for every n, m <= 40, splits them into pairs and passes them as a
 // kernel parameter; each block copies the (P+1)^2 it needs to shared memory.
 
-__host__ __device__ constexpr size_t basis_df_smem_bytes(int P, int warps)
+__host__ __device__ constexpr size_t basis_df_smem_bytes(int P, int groups)
 {
-    // tables a, b ((P+1)^2 each), D, E (P+1 each); per warp: 4 (P+1) state
+    // tables a, b ((P+1)^2 each), D, E (P+1 each); per group: 4 (P+1) state
     // slots x 32 lanes and a 32 x (2P+1) staging tile (8-byte words)
     return 8 * ((size_t)2 * (P + 1) * (P + 1) + (size_t)2 * (P + 1) +
-                (size_t)warps * 32 * ((size_t)4 * (P + 1) + (size_t)(2 * P + 1)));
+                (size_t)groups * 32 * ((size_t)4 * (P + 1) + (size_t)(2 * P + 1)));
 }
 
 struct BasisDfWarp {
@@ -405,65 +435,76 @@ struct BasisDfWarp {
     double *stage;  // [32 rows][2P + 1]
 };
 
-// One group of up to 32 points (rows i0 .. i0 + rows - 1): the degree loop.
-template <bool kChecked>
+// One group of up to 32 points (rows i0 .. i0 + rows - 1), orders wi, wi + S, ...:
+// the degree loop.
+template <bool kChecked, int S>
 __device__ __forceinline__ void basis_df_rows(int P, const float2 *ta, const float2 *tb, const float2 *td,
-                                              const float2 *te, const BasisDfWarp &w, int lane, float2 X,
-                                              float2 Y, float2 Z, float2 R2, int e, int rows, double *og,
+                                              const float2 *te, const BasisDfWarp &w, int sub, int wi, int lane,
+                                              float2 X, float2 Y, float2 Z, float2 R2, int e, int rows, double *og,
                                               int ld)
 {
     const int W = P + 1, pitch = 2 * P + 1;
-    float2 C = make_float2(1.f, 0.f), S = make_float2(0.f, 0.f);  // (x + i y)^n, scaled
+    float2 C = make_float2(1.f, 0.f), T = make_float2(0.f, 0.f);  // (x + i y)^n, scaled
     double *srow = w.stage + lane * pitch;
     for (int n = 0; n <= P; ++n) {
         const int en = e * n;
         const uint32_t kb = (uint32_t)(896 + en) << 20;
         float2 *cur = w.pst + (n & 1) * 32 * W, *prv = w.pst + ((n & 1) ^ 1) * 32 * W;
         double *sc = srow + n;  // column n + m holds the cosine part, n - m the sine part
-        if (n > 0) {
-            const float2 c2 = df_sub(df_mul(C, X), df_mul(S, Y));
-            S = df_add_df(df_mul(S, X), df_mul(C, Y));
-            C = c2;
-        }
-        w.cs[32 * n] = C;
-        w.ss[32 * n] = S;
-        {  // m = n
-            const float2 pd = td[n];
-            cur[32 * n] = pd;
-            sc[n] = df_to_f64_scaled<kChecked>(df_mul(pd, C), kb, en);
-            if (n > 0) sc[-n] = df_to_f64_scaled<kChecked>(df_mul(pd, S), kb, en);
-        }
-        if (n > 0) {  // m = n - 1
-            const int m = n - 1;
-            const float2 p = df_mul(te[m], Z);
-            cur[32 * m] = p;
-            if (m == 0) {
-                sc[0] = df_to_f64_scaled<kChecked>(p, kb, en);
-            } else {
-                sc[m] = df_to_f64_scaled<kChecked>(df_mul(p, w.cs[32 * m]), kb, en);
-                sc[-m] = df_to_f64_scaled<kChecked>(df_mul(p, w.ss[32 * m]), kb, en);
+        if constexpr (S == 1) {
+            if (n > 0) {
+                const float2 c2 = df_sub(df_mul(C, X), df_mul(T, Y));
+                T = df_add_df(df_mul(T, X), df_mul(C, Y));
+                C = c2;
             }
+            w.cs[32 * n] = C;
+            w.ss[32 * n] = T;
+            {  // m = n
+                const float2 pd = td[n];
+                cur[32 * n] = pd;
+                sc[n] = df_to_f64_scaled<kChecked>(df_mul(pd, C), kb, en);
+                if (n > 0) sc[-n] = df_to_f64_scaled<kChecked>(df_mul(pd, T), kb, en);
+            }
+            if (n > 0) {  // m = n - 1
+                const int m = n - 1;
+                const float2 p = df_mul(te[m], Z);
+                cur[32 * m] = p;
+                if (m == 0) {
+                    sc[0] = df_to_f64_scaled<kChecked>(p, kb, en);
+                } else {
+                    sc[m] = df_to_f64_scaled<kChecked>(df_mul(p, w.cs[32 * m]), kb, en);
+                    sc[-m] = df_to_f64_scaled<kChecked>(df_mul(p, w.ss[32 * m]), kb, en);
+                }
+            }
+        } else if (wi == 0 && n < P) {  // the next power: its warp reads it after this degree's barriers
+            const float2 c2 = df_sub(df_mul(C, X), df_mul(T, Y));
+            T = df_add_df(df_mul(T, X), df_mul(C, Y));
+            C = c2;
+            w.cs[32 * (n + 1)] = C;
+            w.ss[32 * (n + 1)] = T;
         }
-        if (n >= 2) {  // m = 0: (x + i y)^0 = 1
-            const float2 pn = df_dot2_sub(ta[n], df_mul(Z, prv[0]), tb[n], df_mul(R2, cur[0]));
+        if (wi == 0 && (S > 1 || n >= 2)) {  // m = 0: (x + i y)^0 = 1
+            const float2 pn = n >= 2   ? df_dot2_sub(ta[n], df_mul(Z, prv[0]), tb[n], df_mul(R2, cur[0]))
+                              : n == 1 ? df_mul(te[0], Z)
+                                       : td[0];
             cur[0] = pn;
             sc[0] = df_to_f64_scaled<kChecked>(pn, kb, en);
         }
         // m >= 1, two orders per pass: their chains are independent, which
         // doubles the instruction-level parallelism of the double-float work
-        int m = 1;
-        for (; m + 3 <= n; m += 2) {
-            const float2 p1a = prv[32 * m], p2a = cur[32 * m], p1b = prv[32 * m + 32], p2b = cur[32 * m + 32];
-            const float2 ca = w.cs[32 * m], sa = w.ss[32 * m], cb = w.cs[32 * m + 32], sb = w.ss[32 * m + 32];
+        int m = wi == 0 ? S : wi;
+        for (; m + S + 2 <= n; m += 2 * S) {
+            const int k = m + S;
+            const float2 p1a = prv[32 * m], p2a = cur[32 * m], p1b = prv[32 * k], p2b = cur[32 * k];
+            const float2 ca = w.cs[32 * m], sa = w.ss[32 * m], cb = w.cs[32 * k], sb = w.ss[32 * k];
             const float2 pa = df_dot2_sub(ta[m * W + n], df_mul(Z, p1a), tb[m * W + n], df_mul(R2, p2a));
-            const float2 pb =
-                df_dot2_sub(ta[(m + 1) * W + n], df_mul(Z, p1b), tb[(m + 1) * W + n], df_mul(R2, p2b));
+            const float2 pb = df_dot2_sub(ta[k * W + n], df_mul(Z, p1b), tb[k * W + n], df_mul(R2, p2b));
             cur[32 * m] = pa;
-            cur[32 * m + 32] = pb;
+            cur[32 * k] = pb;
             sc[m] = df_to_f64_scaled<kChecked>(df_mul(pa, ca), kb, en);
             sc[-m] = df_to_f64_scaled<kChecked>(df_mul(pa, sa), kb, en);
-            sc[m + 1] = df_to_f64_scaled<kChecked>(df_mul(pb, cb), kb, en);
-            sc[-m - 1] = df_to_f64_scaled<kChecked>(df_mul(pb, sb), kb, en);
+            sc[k] = df_to_f64_scaled<kChecked>(df_mul(pb, cb), kb, en);
+            sc[-k] = df_to_f64_scaled<kChecked>(df_mul(pb, sb), kb, en);
         }
         if (m + 2 <= n) {
             const float2 p1 = prv[32 * m], p2 = cur[32 * m];
@@ -471,25 +512,32 @@ __device__ __forceinline__ void basis_df_rows(int P, const float2 *ta, const flo
             cur[32 * m] = pn;
             sc[m] = df_to_f64_scaled<kChecked>(df_mul(pn, w.cs[32 * m]), kb, en);
             sc[-m] = df_to_f64_scaled<kChecked>(df_mul(pn, w.ss[32 * m]), kb, en);
+            m += S;
         }
-        __syncwarp();
+        if (S > 1 && m <= n) {  // m = n or n - 1
+            const float2 pn = m == n ? td[m] : df_mul(te[m], Z);
+            cur[32 * m] = pn;
+            sc[m] = df_to_f64_scaled<kChecked>(df_mul(pn, w.cs[32 * m]), kb, en);
+            sc[-m] = df_to_f64_scaled<kChecked>(df_mul(pn, w.ss[32 * m]), kb, en);
+        }
+        group_sync<S>(sub);
         const int wd = 2 * n + 1, tot = rows * wd;
         const uint32_t cw = ((1u << 20) + (uint32_t)wd - 1u) / (uint32_t)wd;  // ceil(2^20 / (2n + 1))
         double *ob = og + n * n;
 #pragma unroll 4
-        for (int f = lane; f < tot; f += 32) {
+        for (int f = lane + 32 * wi; f < tot; f += 32 * S) {
             const int r = (int)(((uint32_t)f * cw) >> 20), j = f - r * wd;
             ob[r * ld + j] = w.stage[r * pitch + j];
         }
-        __syncwarp();
+        group_sync<S>(sub);
     }
 }
 
-template <int kWarps>
-__global__ void __launch_bounds__(32 * kWarps) basis_df_kernel(const __grid_constant__ BasisDfTables tabs,
-                                                                      int P, double inv_rs, long long np,
-                                                                      const double *__restrict__ pts, int stride,
-                                                                      double *__restrict__ out, long long ld)
+template <int S, int kThreads>
+__global__ void __launch_bounds__(kThreads) basis_df_kernel(const __grid_constant__ BasisDfTables tabs, int P,
+                                                            double inv_rs, long long np,
+                                                            const double *__restrict__ pts, int stride,
+                                                            double *__restrict__ out, long long ld)
 {
     extern __shared__ float2 tab[];
     const int W = P + 1, pitch = 2 * P + 1;
@@ -504,12 +552,12 @@ __global__ void __launch_bounds__(32 * kWarps) basis_df_kernel(const __grid_cons
         te[m] = tabs.e[m];
     }
     __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float2 *wb = te + W + (size_t)warp * 32 * (4 * W + pitch);
+    const int sub = threadIdx.x / (32 * S), wi = (threadIdx.x >> 5) % S, lane = threadIdx.x & 31;
+    const int per_block = blockDim.x / (32 * S);
+    float2 *wb = te + W + (size_t)sub * 32 * (4 * W + pitch);
     const BasisDfWarp w{wb + lane, wb + 64 * W + lane, wb + 96 * W + lane, reinterpret_cast<double *>(wb + 128 * W)};
     const long long ngroups = (np + 31) / 32;
-    for (long long g = (long long)blockIdx.x * (blockDim.x >> 5) + warp; g < ngroups;
-         g += (long long)gridDim.x * (blockDim.x >> 5)) {
+    for (long long g = (long long)blockIdx.x * per_block + sub; g < ngroups; g += (long long)gridDim.x * per_block) {
         const long long i0 = g * 32;
         const int rows = (int)min(32LL, np - i0);
         const long long i = i0 + min(lane, rows - 1);  // lanes past the end repeat the last point, unwritten
@@ -529,9 +577,9 @@ __global__ void __launch_bounds__(32 * kWarps) basis_df_kernel(const __grid_cons
         const bool finite = isfinite(px) && isfinite(py) && isfinite(pz);
         const bool plain = __all_sync(0xffffffffu, finite && abs(e) * P <= 895);
         if (plain)
-            basis_df_rows<false>(P, ta, tb, td, te, w, lane, X, Y, Z, R2, e, rows, out + i0 * ld, (int)ld);
+            basis_df_rows<false, S>(P, ta, tb, td, te, w, sub, wi, lane, X, Y, Z, R2, e, rows, out + i0 * ld, (int)ld);
         else
-            basis_df_rows<true>(P, ta, tb, td, te, w, lane, X, Y, Z, R2, e, rows, out + i0 * ld, (int)ld);
+            basis_df_rows<true, S>(P, ta, tb, td, te, w, sub, wi, lane, X, Y, Z, R2, e, rows, out + i0 * ld, (int)ld);
     }
 }
 
@@ -739,31 +787,60 @@ int launch_quadrature(int F2, int F1, double Rs, double4_32a *dirs, cudaStream_t
     return HSMA_OK;
 }
 
-// Warps per block.  Blocks of two copy the tables often and leave shared
-// memory unused (10 warps per SM at p = 12, 2 from p = 29 on); a larger block
-// is taken where it brings a tenth more warps.  Not 5, 9 or 10 per SM: one or
-// two of its four sub-partitions then have a warp more than the others, which
-// all wait for (p = 25 in double float 829 us with five against 745 with four,
-// p = 14 411 with ten against 395 with eight).  Both forms take the same shared
-// memory; a block has 1 KB of its own.  Measured, in double float: 1e6 points
-// at p = 12 601 -> 544 us, 3e5 at p = 20 543 -> 491, 2e5 at p = 22 523 -> 450,
-// 6e4 at p = 32 619 -> 403; FP64: p = 20 956 -> 870, p = 22 1018 -> 752.
-static int basis_warps(int P, long long groups, int sms)
+// Groups of 32 points per block, and warps that share a group's orders.  A
+// group's state and staging are the same for any number of warps, so where
+// shared memory holds few groups per SM (8 at p = 16, 5 at p = 25, 2 at p = 40),
+// or the call has few, more warps each keep the pipes busier.  Eight for one or
+// two groups per SM (for up to four from p = 28 on), four for up to six from
+// p = 17 on (below, a warp would be left with too few orders), two for the rest
+// of up to eight from p = 17 on, or up to four; one above, where the powers and
+// the barriers of a split cost more than they hide (p = 12, 1e6 points: 591 us
+// with two, 572 with one).  One -> S warps, us, in double float / FP64:
+//   2003 points    p = 12 44 / 57 -> 36 / 37, p = 25 85 / 140 -> 50 / 62
+//   30011 points   p = 25 142 / 258 -> 113 / 176, p = 40 524 / 1103 -> 234 / 458
+//   1e5 points     p = 18 180 / 305 -> 159 / 263, p = 25 361 / 710 -> 264 / 462
+// Four warps a group: blocks of two or four groups where these hold more per SM
+// (p = 20: six instead of five) and the call fills them.
+// With one warp a group, a larger block is taken where it brings a tenth more
+// warps, but not 5, 9 or 10 per SM: one or two of its four sub-partitions then
+// have a warp more than the others, which all wait for (1e6 points at p = 12 601
+// -> 544 us).  Both forms take the same shared memory; a block has 1 KB of its
+// own.
+struct BasisShape {
+    int groups, warps;
+};
+
+static BasisShape basis_shape(int P, long long groups, int sms)
 {
-    auto per_sm = [&](int w) {
-        return w * (int)std::min<size_t>({228 * 1024 / (basis_smem_bytes(P, w) + 1024), (size_t)(64 / w), (size_t)32});
+    auto per_sm = [&](int g) {
+        return g * (int)std::min<size_t>({228 * 1024 / (basis_smem_bytes(P, g) + 1024), (size_t)(64 / g), (size_t)32});
     };
-    int best = 2, most = per_sm(2);
+    int best = 2, most = per_sm(2), hold = most;
     const int two = most;
-    for (int w = 1; w <= kBasisWarps; ++w) {
-        if (w > 2 && groups < (long long)w * sms) break;
-        const int n = per_sm(w);
+    for (int g = 1; g <= kBasisGroups; ++g) {
+        if (g > 2 && groups < (long long)g * sms) break;
+        const int n = per_sm(g);
+        hold = std::max(hold, n);
         if (n > most && 10 * n >= 11 * two && n != 5 && n != 9 && n != 10) {
             most = n;
-            best = w;
+            best = g;
         }
     }
-    return best;
+    const long long resident = std::min<long long>(hold, (groups + sms - 1) / sms);
+    int warps = 1;
+    if (resident <= 2 || (resident <= 4 && P >= 28))
+        warps = 8;
+    else if (P >= 17 && resident <= 6)
+        warps = 4;
+    else if ((P >= 17 && resident <= 8) || resident <= 4)
+        warps = 2;
+    while (warps > 1 && 2 * warps > P + 1) warps /= 2;
+    if (warps == 1) return BasisShape{best, 1};
+    int g = 1;
+    if (warps == 4 && groups > 6LL * sms)
+        for (int k = 2; k <= 4; k += 2)
+            if (per_sm(k) > per_sm(g)) g = k;
+    return BasisShape{g, warps};
 }
 
 int launch_basis(int P, double Rs, long long np, const double *pts, int stride, double *out, long long ld,
@@ -776,14 +853,18 @@ int launch_basis(int P, double Rs, long long np, const double *pts, int stride, 
     HSMA_CUDA_TRY(cudaGetDevice(&dev));
     HSMA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const long long groups = (np + 31) / 32;
-    const int warps = basis_warps(P, groups, sms);
-    const size_t smem = basis_smem_bytes(P, warps);
-    auto kernel = warps <= 2 ? basis_kernel<2> : basis_kernel<kBasisWarps>;
+    const BasisShape sh = basis_shape(P, groups, sms);
+    const size_t smem = basis_smem_bytes(P, sh.groups);
+    auto kernel = sh.warps == 1   ? (sh.groups <= 2 ? basis_kernel<1, 64> : basis_kernel<1, 32 * kBasisGroups>)
+                  : sh.warps == 2 ? basis_kernel<2, 64>
+                  : sh.warps == 4 ? basis_kernel<4, 512>
+                                  : basis_kernel<8, 256>;
     HSMA_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    HSMA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32 * warps, smem));
+    const int threads = 32 * sh.groups * sh.warps;
+    HSMA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
     if (per_sm < 1) return HSMA_E_ARG;
-    const long long blocks = std::min<long long>((groups + warps - 1) / warps, (long long)sms * per_sm);
-    kernel<<<(unsigned)blocks, 32 * warps, smem, st>>>(basis_f64_tables(), P, 1.0 / Rs, np, pts, stride, out, (int)ld);
+    const long long blocks = std::min<long long>((groups + sh.groups - 1) / sh.groups, (long long)sms * per_sm);
+    kernel<<<(unsigned)blocks, threads, smem, st>>>(basis_f64_tables(), P, 1.0 / Rs, np, pts, stride, out, (int)ld);
     HSMA_LAUNCHED();
     HSMA_CUDA_TRY(cudaGetLastError());
     return HSMA_OK;
@@ -799,14 +880,18 @@ int launch_basis_df(int P, double Rs, long long np, const double *pts, int strid
     HSMA_CUDA_TRY(cudaGetDevice(&dev));
     HSMA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const long long groups = (np + 31) / 32;
-    const int warps = basis_warps(P, groups, sms);
-    const size_t smem = basis_df_smem_bytes(P, warps);
-    auto kernel = warps <= 2 ? basis_df_kernel<2> : basis_df_kernel<kBasisWarps>;
+    const BasisShape sh = basis_shape(P, groups, sms);
+    const size_t smem = basis_df_smem_bytes(P, sh.groups);
+    auto kernel = sh.warps == 1   ? (sh.groups <= 2 ? basis_df_kernel<1, 64> : basis_df_kernel<1, 32 * kBasisGroups>)
+                  : sh.warps == 2 ? basis_df_kernel<2, 64>
+                  : sh.warps == 4 ? basis_df_kernel<4, 512>
+                                  : basis_df_kernel<8, 256>;
     HSMA_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    HSMA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32 * warps, smem));
+    const int threads = 32 * sh.groups * sh.warps;
+    HSMA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
     if (per_sm < 1) return HSMA_E_ARG;
-    const long long blocks = std::min<long long>((groups + warps - 1) / warps, (long long)sms * per_sm);
-    kernel<<<(unsigned)blocks, 32 * warps, smem, st>>>(basis_df_tables(), P, 1.0 / Rs, np, pts, stride, out, ld);
+    const long long blocks = std::min<long long>((groups + sh.groups - 1) / sh.groups, (long long)sms * per_sm);
+    kernel<<<(unsigned)blocks, threads, smem, st>>>(basis_df_tables(), P, 1.0 / Rs, np, pts, stride, out, ld);
     HSMA_LAUNCHED();
     HSMA_CUDA_TRY(cudaGetLastError());
     return HSMA_OK;
