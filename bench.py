@@ -42,7 +42,7 @@ RECIPE_MAX_SM_MHZ = 2070.0
 # keyed by (N, pair variant, items per slot) of the captured launch.
 PAIR_FP32_TRAFFIC_BYTES = {(100_000, 17, 48): 361.16e6, (100_000, 14, 48): 356.89e6,
                            (100_000, 17, 96): 726.99e6, (100_000, 14, 96): 710.68e6}
-OPS_SURFACE = 45                 # FP32 lane instructions per particle-direction pair of the surface kernel
+OPS_SURFACE = 24                 # FP32 lane instructions per particle-direction pair of the surface kernel
 
 
 def parse():
@@ -881,7 +881,7 @@ def main():
                                         "frac_of_scalar_fma": achieved / fp32_meas[0],
                                         "how": "hsma_fp32_peak: register-only FMA chains, 16 CTAs/SM"}
                                        if fp32_meas else None)},
-        "roofline_surface": {"bound": "alu", "kernel": "surface_pairs_fp32_kernel",
+        "roofline_surface": {"bound": "alu", "kernel": "surface_dipole_fp32_kernel",
                              "achieved": OPS_SURFACE * pairs_surf / (phases[5] / 1000.0) / 1e12,
                              "peak": peak_ops / 1e12, "unit": "T FP32 lane-instructions/s",
                              "frac": OPS_SURFACE * pairs_surf / (phases[5] / 1000.0) / peak_ops,
