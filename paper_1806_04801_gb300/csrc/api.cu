@@ -291,9 +291,10 @@ hsma_tuning choose_tuning(const hsma_plan_s *p, int nsys, const long long *n)
     }
     if (best) return *best;
     // untuned FP32: packed variants, two targets per thread where blocks of 384
-    // leave the chip with too few items (step time with 13 / 17 / 14: N = 500
-    // 219 / 224 / 246 us, N = 1000 241 / 257 / 257), three above (N = 4000 451 /
-    // 452 / 486, N = 8000 843 / 815 / 947, N = 16000 2132 / 2117 / 2248)
+    // leave the chip with too few items (step time with 13 / 17, p = 10: N = 400
+    // 144 / 159 us, N = 1000 170 / 186), three above (N = 2000 234 / 236, N = 4000
+    // 400 / 379, N = 8000 798 / 757, N = 30000 6083 / 6002; 14 was up to 16% slower
+    // than 17 up to N = 16000); 1e8 pairs are N = 1600 there
     if (p->precision == HSMA_FP64) return hsma_tuning{4, 24, 0.0};
     return hsma_tuning{batch_work(p, nsys, n) < 1e8 ? 13 : 17, 48, 0.0};
 }
