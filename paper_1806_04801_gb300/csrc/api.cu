@@ -330,8 +330,12 @@ void shape_batch(const hsma_plan_s *p, int nsys, const long long *n, int precisi
     // two -> eight: FP64 N = 1000 562 -> 527 us, N = 2000 1174 -> 1079, grounded
     // N = 3001 1970 -> 1900; FP32 variant 17 N = 4000 392 -> 379, N = 8000 775 ->
     // 757; sixteen is slower from N = 8000 on, FP32 N >= 16000 alike)
+    // -- in FP64, whose pairs take longer, twenty-four (eight -> twenty-four:
+    // periodic N = 2500 1421 -> 1386 us, N = 5000 3768 -> 3640, grounded N = 3001
+    // 1891 -> 1854; N = 1000, and from 8000 on, within 1%)
+    const double least = precision == HSMA_FP64 ? 24.0 : 8.0;
     const double chunk =
-        std::max(std::min(4.0 * tile, std::max(1.0 * tile, work / (8.0 * slots))), work / items_wanted);
+        std::max(std::min(4.0 * tile, std::max(1.0 * tile, work / (least * slots))), work / items_wanted);
     long long part = 0, src = 0, tgt = 0, rec = 0, cnt = 0, hist = 0, tiles = 0, max_tiles = 0;
     long long items = 0, surf = 0;
     int nblk_max = 1;
