@@ -533,15 +533,18 @@ __global__ void __launch_bounds__(kThreads, MINB) pair_fp32_kernel(PairArgs a)
 // (1.96e9 pairs) 61.3 -> 10.5 ms, 3.2e10 -> 1.87e11 pairs/s; N = 1000 1.30 ->
 // 0.22 ms; grounded N = 3001 9.4 -> 1.56 ms.  Error against quad
 // precision (N = 300..4000, both boundaries, three charge patterns): field
-// 1.6e-16..8.0e-16 of its norm against 4.7e-16..1.7e-15 before, potential
-// 1.5e-16..3.9e-15 against 3.5e-16..5.2e-15.
+// 1.8e-16..1.2e-15 of its norm against 4.7e-16..1.7e-15 before, potential
+// 1.4e-16..3.9e-15 against 3.5e-16..5.2e-15.  Those have charges of like size;
+// a tile with one far above the others goes native (fx_charges_fit; normal
+// charges now and then, and in a last tile of less than about 80: 527 -> 543 us
+// for 20011 sources x 3001 targets).
 struct FxShared {
     double4_32a src[2][kTile64];       // staged sources (bulk copies land here)
     FxSource fx[kTile64];              // the tile being summed, in fixed point
     double tgt[kT64][3][kThreads];     // this block's targets
     double acc[kT64][4][kThreads];     // their potential and field sums
     float2 gf[kT64][3][kThreads];      // double-float sums of FxSums::gf of a tile
-    unsigned qmax[2][kThreads / 32], qmin[2][kThreads / 32];
+    unsigned qmax[kThreads / 32], tally[kThreads / 32];
 };
 
 // |v| as the upper word of its bits (ordered like |v|).
@@ -815,9 +818,9 @@ __global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
                 const long long o = part && tidx[t] >= 0 ? tidx[t] - s0 : -1;
                 self_rel[t] = o >= 0 && o < kTile64 ? (int)o : -1;
             }
-            // charge range of the tile; 0x7fffffff marks what the formats do not
+            // largest charge of the tile; 0x7fffffff marks what the formats do not
             // hold.  The coordinates are converted on the way.
-            unsigned qmax = 0u, qmin = 0x7fffffffu;
+            unsigned qmax = 0u;
             for (int s = tid; s < cnt; s += kThreads) {
                 const double4_32a p = sm.src[buf][s];
                 FxSource &f = sm.fx[s];
@@ -827,34 +830,33 @@ __global__ void __launch_bounds__(kThreads, 4) pair_fp64_kernel(PairArgs a)
                 ok = split(p.y, 1, src_lim, f.hy, f.ly, f.fy) && ok;
                 ok = split(p.z, 2, src_lim, f.hz, f.lz, f.fz) && ok;
                 qmax = max(qmax, ok ? hq : 0x7fffffffu);
-                if (p.w != 0.0) qmin = min(qmin, hq);
             }
             qmax = __reduce_max_sync(0xffffffffu, qmax);
-            qmin = __reduce_min_sync(0xffffffffu, qmin);
-            if (lane == 0) {
-                sm.qmax[buf][wid] = qmax;
-                sm.qmin[buf][wid] = qmin;
-            }
+            if (lane == 0) sm.qmax[wid] = qmax;
             __syncthreads();
             if (s_abort) break;
 #pragma unroll
-            for (int w = 0; w < kThreads / 32; ++w) {
-                qmax = max(qmax, sm.qmax[buf][w]);
-                qmin = min(qmin, sm.qmin[buf][w]);
-            }
-            // the largest |q| scaled to [1/2, 1); the smallest must keep its
-            // bits next to it (a target that skips the largest sees only the others)
-            int eq = qmax == 0u ? 1022 : (int)(qmax >> 20);
-            const bool native =
-                blk_native || eq > 1923 || eq < 123 || (qmax != 0u && (int)(qmin >> 20) < eq - 20);
+            for (int w = 0; w < kThreads / 32; ++w) qmax = max(qmax, sm.qmax[w]);
+            // the largest |q| scaled to [1/2, 1)
+            const int eq = qmax == 0u ? 1022 : (int)(qmax >> 20);
+            bool native = blk_native || eq > 1923 || eq < 123;
             if (!native) {
                 for (int s = cnt + tid; s < (cnt + kStepFx - 1) / kStepFx * kStepFx; s += kThreads)
                     sm.fx[s] = FxSource{src_lim, src_lim, src_lim, 0, 0, 0, 0, 0u, 0.f, 0.f, 0.f, 0.f};
+                unsigned tally = 0u;
                 for (int s = tid; s < cnt; s += kThreads) {
-                    fx_split_charge(fx_fixed(sm.src[buf][s].w, 63 + 1022 - eq), sm.fx[s].qh, sm.fx[s].ql,
-                                    sm.fx[s].fq);
+                    const double q = sm.src[buf][s].w;
+                    FxSource &f = sm.fx[s];
+                    fx_split_charge(fx_fixed(q, 63 + 1022 - eq), f.qh, f.ql, f.fq);
+                    tally += fx_charge_tally(f.fq, abs_hi(q) != 0u);
                 }
+                tally = __reduce_add_sync(0xffffffffu, tally);
+                if (lane == 0) sm.tally[wid] = tally;
                 __syncthreads();
+                tally = 0u;
+#pragma unroll
+                for (int w = 0; w < kThreads / 32; ++w) tally += sm.tally[w];
+                native = !fx_charges_fit(tally, qmax == 0u ? 0u : (0x100000u | (qmax & 0xfffffu)) >> 7);
             }
             if (native || native_tiles > 0) {
                 --native_tiles;
