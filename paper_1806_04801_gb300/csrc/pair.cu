@@ -652,7 +652,6 @@ __device__ __forceinline__ int tile_fx(FxShared &sm, int buf, int cnt, const FxT
                 sums[t].gf[c] = 0.f;
             }
     };
-    auto near = [](uint64_t A) { return (uint32_t)(A >> 32) < (uint32_t)(kFxNearA >> 32); };
     // kStepFx sources per step: one branch for their near pairs, and
     // independent chains to issue (the slots past cnt hold uncharged sources)
 #pragma unroll 1
@@ -673,7 +672,7 @@ __device__ __forceinline__ int tile_fx(FxShared &sm, int buf, int cnt, const FxT
                 dh[i][t][2] = f.hz - tg[t].h[2];
                 const int dl[3] = {f.lx - tg[t].l[0], f.ly - tg[t].l[1], f.lz - tg[t].l[2]};
                 A[i][t] = fx_distance2(dh[i][t], dl);
-                any = any || near(A[i][t]);
+                any = any || fx_near(A[i][t]);
             }
         }
         if (any) {
@@ -685,7 +684,7 @@ __device__ __forceinline__ int tile_fx(FxShared &sm, int buf, int cnt, const FxT
                     uint64_t Ai = A[0][t];
 #pragma unroll
                     for (int j = 1; j < kStepFx; ++j) Ai = i == j ? A[j][t] : Ai;
-                    if (near(Ai)) {
+                    if (fx_near(Ai)) {
                         ++slow;
                         pair64<FIELD>(p, sm.tgt[t][0][tid], sm.tgt[t][1][tid], sm.tgt[t][2][tid],
                                       s0 + i == self_rel[t], skip_zero, sm.acc[t][0][tid], sm.acc[t][1][tid],
@@ -700,7 +699,7 @@ __device__ __forceinline__ int tile_fx(FxShared &sm, int buf, int cnt, const FxT
             const float fq = f.fq;
 #pragma unroll
             for (int t = 0; t < kT64; ++t) {
-                const FxPair r = fx_inverse(A[i][t], near(A[i][t]), f.qh, f.ql);
+                const FxPair r = fx_inverse(A[i][t], fx_near(A[i][t]), f.qh, f.ql);
                 fx_add_potential(sums[t], r, fq);
                 if (FIELD) {
                     const float df[3] = {f.fx - tg[t].f[0], f.fy - tg[t].f[1], f.fz - tg[t].f[2]};

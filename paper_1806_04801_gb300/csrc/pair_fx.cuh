@@ -214,6 +214,12 @@ HSMA_HD uint64_t fx_distance2(const int (&dh)[3], const int (&dl)[3])
     return a + (uint64_t)(b >> 29);
 }
 
+// Whether a pair at this distance^2 is nearer than kFxNearR.  fx_distance2
+// leaves out sum dl^2 (below eight units), so that two points within a unit of
+// the high words can get a small negative number: its high word, all ones,
+// becomes the smallest here.  (No true distance^2 reaches it: at most 12 2^60.)
+HSMA_HD bool fx_near(uint64_t A) { return (uint32_t)(A >> 32) + 1u < (uint32_t)(kFxNearA >> 32) + 1u; }
+
 struct FxPair {
     int64_t q0;        // q y, units 2^-59
     int64_t x;         // q y (3 e/2 + 15 e^2/8), the same units
