@@ -1576,6 +1576,13 @@ int hsma_plan_set_inset_skin(hsma_plan_t pl, double skin)
         pl->md_nshifts = (int)sh.size();
         pl->md_shifts_dirty = true;
     }
+    if (skin != pl->md_skin) {
+        // the captured launches hold the skin (candidates' radius and shifts,
+        // stale test, ranges) and the list's arrays, which move with the
+        // number of shifts
+        cudaStreamSynchronize(pl->stream ? pl->stream : pl->priv_stream);
+        drop_graphs(pl);
+    }
     pl->md_skin = skin;
     pl->md_valid = false;
     return HSMA_OK;
