@@ -697,18 +697,19 @@ int work_stream(hsma_plan_s *p, cudaStream_t *out)
     return HSMA_OK;
 }
 
-// Device memory of the reusable in-set for systems of n particles.
+// Device memory of the reusable in-set for systems of n particles.  The shift
+// table comes first: it is written once per skin, not once per n.
 size_t carve_md(hsma_plan_s *p, long long n, void *base)
 {
     const long long nblk = (n + kInsetBlock - 1) / kInsetBlock;
     Carver c(base);
+    p->md_shifts = c.take<int4>(p->md_nshifts);
     p->md_cand = c.take<int2>((size_t)n * p->md_nshifts);
     p->md_perm = c.take<int>(n);
     p->md_x0 = c.take<double4_32a>(n);
     p->md_u = c.take<double4_32a>(n);
     p->md_counts = c.take<int>((size_t)p->md_nshifts * nblk);
     p->md_rcounts = c.take<int>((size_t)p->md_nshifts * nblk + 1);  // per block of 256 candidates
-    p->md_shifts = c.take<int4>(p->md_nshifts);
     p->md_ns = c.take<long long>(1);
     return align_up(c.off, 256);
 }
