@@ -586,7 +586,8 @@ int enqueue_update(hsma_plan_s *p, const BatchShape &sh, const Workspace &w, int
     ia.cen = w.cen;
     ia.cenf = w.cenf;
     ia.qsums = w.qsums;
-    if ((rc = small ? launch_inset_small(ia, st) : launch_inset(ia, st))) return rc;
+    const bool few_counts = (long long)ia.n_shifts * ia.nblk_max <= kSmallCounts;
+    if ((rc = small && few_counts ? launch_inset_small(ia, st) : launch_inset(ia, st))) return rc;
     if (mode == kBuild) {
         // candidates within Rs + skin over the enlarged shift table, and the
         // order and positions they refer to

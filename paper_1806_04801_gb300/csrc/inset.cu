@@ -187,8 +187,8 @@ __device__ __forceinline__ void check_neutral(const InsetArgs &a, const SysDesc 
 }
 
 // SCANNED: a.counts holds the exclusive prefix; otherwise the counts, whose
-// prefix every block adds up for itself (small systems: at most 16 blocks per
-// shift), the last one also the total.
+// prefix every block adds up for itself (at most kSmallCounts of them), the
+// last one also the total.
 template <bool SCANNED>
 __global__ void __launch_bounds__(kInsetThreads) inset_scatter_kernel(InsetArgs a)
 {
