@@ -423,8 +423,13 @@ void hsma_server_destroy(hsma_server_t srv);
  * over ns sources (src: ns x 4 doubles x, y, z, q) and nt targets (tgt:
  * nt x 3), all device pointers.  A pair at distance exactly 0 is skipped.
  * field may be NULL.  precision as in hsma_precision (0 or 1).
- * stream: cudaStream_t or NULL.  Errors: HSMA_E_ARG, HSMA_E_OOM,
- * HSMA_E_CUDA. */
+ * stream: cudaStream_t or NULL.
+ * Working memory -- about 32 (ns + nt) bytes and up to 160 MB of partial sums --
+ * comes from the device's default memory pool.  Above 256 MiB it is given back
+ * before the call returns; up to that the pool keeps it for a next call until
+ * the process next synchronises (a stream, an event or the device).  Calls that
+ * overlap each take their own.
+ * Errors: HSMA_E_ARG, HSMA_E_OOM, HSMA_E_CUDA. */
 int hsma_coulomb_sum(int64_t ns, const double *src, int64_t nt, const double *tgt, double *pot,
                      double *field, int precision, void *stream);
 

@@ -1,0 +1,31 @@
+"""The direct sum's working memory after the call: all of it given back where it is large, a bounded part kept for the
+next call, until the program's next synchronisation, where it is small."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+MIB = 1 << 20
+
+
+# 32 bytes a source and up to 60 MB of partial sums: 9e6 sources need about 350 MB, 1e5 x 5e4 at most 160 MB.
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("ns,nt,keep", [(9_000_000, 1000, 0), (100_000, 50_000, 256 * MIB), (1000, 500, 32 * MIB)])
+def test_direct_sum_keeps_little_memory(ns, nt, keep, precision):
+    import torch
+
+    from paper_1806_04801_gb300 import hsma
+
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    src = torch.rand((ns, 4), generator=g, device="cuda", dtype=torch.float64)
+    tgt = torch.rand((nt, 3), generator=g, device="cuda", dtype=torch.float64)
+    for stream in (torch.cuda.current_stream(), torch.cuda.Stream()):
+        with torch.cuda.stream(stream):
+            hsma.coulomb_sum(src, tgt, precision=precision)  # loads the kernels, makes the results' blocks
+            torch.cuda.synchronize()
+            before = torch.cuda.mem_get_info()[0]
+            for _ in range(3):
+                hsma.coulomb_sum(src, tgt, precision=precision)
+            assert before - torch.cuda.mem_get_info()[0] <= keep
+            torch.cuda.synchronize()
+            assert torch.cuda.mem_get_info()[0] >= before
