@@ -648,7 +648,7 @@ int enqueue_update(hsma_plan_s *p, const BatchShape &sh, const Workspace &w, int
                            p->mon_inv, w.b, w.A, w.tc_work, w.status, fit_ctas(p), st);
     else
         rc = launch_fit_fp64(w.sys, nsys, p->bc, p->K, p->ncols, p->Nb, p->Mp, w.phi_tgt, p->mon_inv, w.b, w.A,
-                             st);
+                             p->num_sms, st);
     if (rc) return rc;
     record(p, st, 4);
 
@@ -667,7 +667,7 @@ int enqueue_update(hsma_plan_s *p, const BatchShape &sh, const Workspace &w, int
         record(p, st, 5);
         if ((rc = launch_surface_pairs(w.sys, nsys, sh.surf_items, w.src_hi, w.src_lo, w.src64, p->ndir,
                                        p->dirs, p->dirs32, w.img, p->Rs, p->R0 + p->md_skin, p->dr, prec, w.phi_out,
-                                       w.e_out, st)))
+                                       w.e_out, p->num_sms, st)))
             return rc;
         record(p, st, 6);
     }
@@ -1098,7 +1098,8 @@ int run_shard(hsma_plan_s *p, const hsma_particles *x, bool far_stage, int part,
             rc = launch_fit_tc(w.sys, 1, p->bc, p->K, p->ncols, p->Nb, p->tc_hi, p->tc_lo, p->tc_mdf, w.phi_tgt,
                                p->mon_inv, w.b, w.A, w.tc_work, w.status, fit_ctas(p), st);
         else
-            rc = launch_fit_fp64(w.sys, 1, p->bc, p->K, p->ncols, p->Nb, p->Mp, w.phi_tgt, p->mon_inv, w.b, w.A, st);
+            rc = launch_fit_fp64(w.sys, 1, p->bc, p->K, p->ncols, p->Nb, p->Mp, w.phi_tgt, p->mon_inv, w.b, w.A,
+                                p->num_sms, st);
         if (rc) return rc;
         if (p->far_field == 1) {
             rc = launch_series_field(w.sys, 1, std::max<long long>(cnt, 1), p->P, p->Rs, p->norm, w.A, w.src_hi,
@@ -1108,7 +1109,7 @@ int run_shard(hsma_plan_s *p, const hsma_particles *x, bool far_stage, int part,
             if (!rc && sh.surf_items > 0)
                 rc = launch_surface_pairs(w.sys, 1, sh.surf_items, w.src_hi, w.src_lo, w.src64, p->ndir,
                                           p->dirs, p->dirs32, w.img, p->Rs, p->R0 + p->md_skin, p->dr, prec, w.phi_out,
-                                          w.e_out, st);
+                                          w.e_out, p->num_sms, st);
         }
         if (rc) return rc;
         // the near stage's Phi_in, E_in of the owned particles into their

@@ -493,7 +493,7 @@ int launch_partial_reduce(const SysDesc *sys, int nsys, long long max_tgt, int n
 // mon_inv[i]: slot of monitoring target i among the (spatially ordered)
 // external targets the pair kernel used, or null for the identity.
 int launch_fit_fp64(const SysDesc *sys, int nsys, int bc, int K, int ncols, int Nb, const double *Mp,
-                    const double *phi_tgt, const int *mon_inv, double *b_out, double *A, cudaStream_t st);
+                    const double *phi_tgt, const int *mon_inv, double *b_out, double *A, int num_sms, cudaStream_t st);
 // f32: img holds float2 pairs (for the FP32 surface sums)
 int launch_surface_charges(int nsys, int ndir, int Nb, const double *Bq, const double4_32a *dirs, const double *A,
                            double Rs, bool f32, double2 *img, cudaStream_t st);
@@ -503,7 +503,7 @@ int launch_directions_fp32(int n, const double4_32a *dirs, float4 *out, cudaStre
 int launch_surface_pairs(const SysDesc *sys, int nsys, int total_items, const float4 *src_hi, const float4 *src_lo,
                          const double4_32a *src64, int ndir, const double4_32a *dirs, const float4 *dirs32,
                          const double2 *img, double Rs, double r_max, double dr, int precision, double *phi_out,
-                         double *e_out, cudaStream_t st);
+                         double *e_out, int num_sms, cudaStream_t st);
 int launch_series_field(const SysDesc *sys, int nsys, long long max_n, int P, double Rs, const double *norm,
                         const double *A, const float4 *src_hi, const float4 *src_lo, const double4_32a *src64,
                         double *phi_out, double *e_out, cudaStream_t st);

@@ -690,9 +690,9 @@ __global__ void __launch_bounds__(kFinalThreads) finalize_kernel(const SysDesc *
 }  // namespace
 
 int launch_fit_fp64(const SysDesc *sys, int nsys, int bc, int K, int ncols, int Nb, const double *Mp,
-                    const double *phi_tgt, const int *mon_inv, double *b_out, double *A, cudaStream_t st)
+                    const double *phi_tgt, const int *mon_inv, double *b_out, double *A, int num_sms, cudaStream_t st)
 {
-    if ((long long)ncols * nsys <= 1216)  // a block per row fills the chip
+    if ((long long)ncols * nsys <= 8LL * num_sms)  // a block per row, at most eight per SM: all resident at once
         fit_fp64_kernel<8><<<dim3(ncols, nsys), 256, 0, st>>>(sys, bc, K, ncols, Nb, Mp, phi_tgt, mon_inv, b_out, A);
     else
         fit_fp64_kernel<1><<<dim3((ncols + 7) / 8, nsys), 256, 0, st>>>(sys, bc, K, ncols, Nb, Mp, phi_tgt, mon_inv,
@@ -717,7 +717,7 @@ int surface_targets_per_block() { return kSurfTB; }
 int launch_surface_pairs(const SysDesc *sys, int nsys, int total_items, const float4 *src_hi, const float4 *src_lo,
                          const double4_32a *src64, int ndir, const double4_32a *dirs, const float4 *dirs32,
                          const double2 *img, double Rs, double r_max, double dr, int precision, double *phi_out,
-                         double *e_out, cudaStream_t st)
+                         double *e_out, int num_sms, cudaStream_t st)
 {
     if (total_items <= 0) return HSMA_OK;
     const double h = 0.5 * dr, rho = Rs - r_max;  // rho: a lower bound
@@ -736,7 +736,7 @@ int launch_surface_pairs(const SysDesc *sys, int nsys, int total_items, const fl
         };
         const bool h2 = h > 3e-5 * rho;
         // blocks of 64 particles from the size where they are two per SM
-        if (total_items >= 304)
+        if (total_items >= 2 * num_sms)
             launch(h2 ? surface_dipole_fp32_kernel<8, 2, true> : surface_dipole_fp32_kernel<8, 2, false>, 64);
         else
             launch(h2 ? surface_dipole_fp32_kernel<32, 1, true> : surface_dipole_fp32_kernel<32, 1, false>, 8);
