@@ -15,6 +15,23 @@ namespace hsma {
 
 namespace {
 
+// Lifts a kernel's limit of dynamic shared memory to the most the device allows
+// beside its static part (an error where `bytes` is more).  The limit belongs to
+// the kernel: set to the call's own size, it made a larger launch of another
+// thread fail in between.
+template <class K>
+cudaError_t allow_smem(K kernel, size_t bytes)
+{
+    int dev = 0, most = 0;
+    cudaFuncAttributes a;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (!e) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (!e) e = cudaFuncGetAttributes(&a, kernel);
+    if (e) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)std::max((size_t)most - a.sharedSizeBytes, bytes));
+}
+
 constexpr double kPi = 3.14159265358979323846;
 
 __device__ __forceinline__ void write_target(long long i, double x, double y, double z, double4_32a *o64, float4 *hi,
@@ -859,7 +876,7 @@ int launch_basis(int P, double Rs, long long np, const double *pts, int stride, 
                   : sh.warps == 2 ? basis_kernel<2, 64>
                   : sh.warps == 4 ? basis_kernel<4, 512>
                                   : basis_kernel<8, 256>;
-    HSMA_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    HSMA_CUDA_TRY(allow_smem(kernel, smem));
     const int threads = 32 * sh.groups * sh.warps;
     HSMA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
     if (per_sm < 1) return HSMA_E_ARG;
@@ -886,7 +903,7 @@ int launch_basis_df(int P, double Rs, long long np, const double *pts, int strid
                   : sh.warps == 2 ? basis_df_kernel<2, 64>
                   : sh.warps == 4 ? basis_df_kernel<4, 512>
                                   : basis_df_kernel<8, 256>;
-    HSMA_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    HSMA_CUDA_TRY(allow_smem(kernel, smem));
     const int threads = 32 * sh.groups * sh.warps;
     HSMA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
     if (per_sm < 1) return HSMA_E_ARG;
@@ -943,11 +960,11 @@ int build_pseudo_inverse(int K, int n, double *Wcol, double *Mp, double *cond_ho
         HSMA_LAUNCHED();
     }
     size_t smq = (size_t)K * sizeof(double);
-    HSMA_CUDA_TRY(cudaFuncSetAttribute(qr_form_q_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smq));
+    HSMA_CUDA_TRY(allow_smem(qr_form_q_kernel, smq));
     qr_form_q_kernel<<<n, 256, smq, st>>>(Wcol, K, n, vtop, vv, Q1);
     HSMA_LAUNCHED();
     size_t smr = (size_t)n * sizeof(double);
-    HSMA_CUDA_TRY(cudaFuncSetAttribute(r_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr));
+    HSMA_CUDA_TRY(allow_smem(r_inverse_kernel, smr));
     r_inverse_kernel<<<n, 128, smr, st>>>(Wcol, K, n, diag, Rinv);
     HSMA_LAUNCHED();
     long long tot = (long long)n * K;
