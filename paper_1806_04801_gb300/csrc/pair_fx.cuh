@@ -187,22 +187,23 @@ HSMA_HD uint32_t fx_charge_tally(float fq, bool nonzero)
 // of fx_charge_tally, largest: the largest |q| in the same units 2^-14.
 //
 // The tally counts without the largest charge, which a target may skip (its own
-// slot, or a source at the target): the others must add up to 16 and to a
-// twelfth each.  Rms error of such a target's sums, fixed point against the
-// FP64 loop (random positions, near pairs left out; potential, field):
-//   256 charges +-1                  0.12, 0.44      64  0.24, 0.74     16  0.42, 0.96
-//   256 normal charges               0.42, 0.74      64  0.70, 1.19     16  1.13, 1.26
-//   1 and 255 charges +-1/4, 1/8     0.13, 0.60 and 1.04, 1.27 (refused), 1/16  3.1, 3.9 (refused)
+// slot, or a source at the target): the others must be 3/8 on average, or add up
+// to 16 and to a twelfth each.  Rms error of such a target's sums, fixed point
+// against the FP64 loop (random positions, near pairs left out; potential, field):
+//   256 charges +-1       0.12, 0.44     64  0.24, 0.74     16  0.42, 0.84     2  0.80, 0.97
+//   256 normal charges    0.42, 0.74     64  0.70, 1.19     16  1.13, 1.26 (mostly refused)
+//   1 and 255 charges +-1/4, 1/8         0.13, 0.60 and 1.04, 1.27 (refused)
+//   1 and 255 charges +-1/16             3.1, 3.9 (refused)
 // (the FP64 loop rounds its running sum at every source, the integers never do,
-// which is what the accuracy of many like charges comes from).  Tiles of 256
+// which is what the accuracy of many unlike charges comes from).  Tiles of 256
 // normal charges pass while their largest is below 4.8 sigma (all but four in
 // 10^4): the scale, a power of two, is then below twelve times their mean.
 HSMA_HD bool fx_charges_fit(uint32_t tally, uint32_t largest)
 {
     const uint32_t nonzero = tally >> 23;
     if (nonzero == 0u) return true;
-    const uint32_t others = (tally & 0x7fffffu) - largest;
-    return others >= 16u << 14 && 12u * others >= (nonzero - 1u) << 14;
+    const uint32_t others = (tally & 0x7fffffu) - largest, each = (nonzero - 1u) << 14;
+    return 8u * others >= 3u * each || (others >= 16u << 14 && 12u * others >= each);
 }
 
 // dh, dl: source minus target.  The distance^2 in units 2^-60.

@@ -37,6 +37,7 @@ int main(int argc, char **argv)
             if (!strcmp(dist, "ions")) q[i] = i % 2 ? par : -par;
             if (!strcmp(dist, "heavy")) q[i] = i == 0 ? 1.0 : sign() * par;  // one charge 1, the others +-par
             if (!strcmp(dist, "lognormal")) q[i] = sign() * std::exp(par * normal(g));
+            if (!strcmp(dist, "uniform")) q[i] = par * u(g);
             if (!strcmp(dist, "zeros")) q[i] = i % 4 ? 0.0 : sign() * (1.0 + par * u(g));
         }
         const int big = (int)(std::max_element(q.begin(), q.end(), [](double a, double b) {

@@ -1,5 +1,5 @@
-"""Harmonic basis from several threads at once: calls whose blocks take different amounts of shared memory share a kernel,
-and its limit."""
+"""Harmonic basis from several threads at once: calls whose blocks take different amounts of shared memory
+share a kernel, and its limit."""
 import threading
 
 import pytest

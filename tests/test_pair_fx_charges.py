@@ -34,8 +34,10 @@ def run(tmp_path_factory):
     ("normal", 256, 1.0, (0.95, 1.0)), ("normal", 256, 1.2e-19, (0.95, 1.0)), ("normal", 200, 1.7, (0.95, 1.0)),
     ("ions", 256, 1.0, (1.0, 1.0)), ("ions", 40, 3.0, (1.0, 1.0)), ("zeros", 256, 0.3, (1.0, 1.0)),
     ("heavy", 256, 0.5, (1.0, 1.0)), ("heavy", 256, 0.25, (1.0, 1.0)), ("lognormal", 256, 0.5, (0.9, 1.0)),
-    ("lognormal", 256, 1.0, (0.0, 1.0)), ("normal", 16, 1.0, (0.0, 0.0)), ("heavy", 256, 2.0**-4, (0.0, 0.0)),
-    ("heavy", 256, 2.0**-10, (0.0, 0.0)), ("heavy", 256, 2.0**-19, (0.0, 0.0)), ("lognormal", 256, 4.0, (0.0, 0.0))])
+    ("lognormal", 256, 1.0, (0.0, 1.0)), ("normal", 16, 1.0, (0.0, 0.3)), ("ions", 2, 1.0, (1.0, 1.0)),
+    ("ions", 13, 1.0, (1.0, 1.0)), ("uniform", 8, 1.0, (0.0, 1.0)), ("zeros", 60, 0.3, (1.0, 1.0)),
+    ("heavy", 256, 2.0**-4, (0.0, 0.0)), ("heavy", 256, 2.0**-10, (0.0, 0.0)), ("heavy", 256, 2.0**-19, (0.0, 0.0)),
+    ("heavy", 12, 0.25, (0.0, 0.0)), ("lognormal", 256, 4.0, (0.0, 0.0))])
 def test_target_that_skips_the_largest_charge(run, dist, n, par, taken):
     accepted, rms_p, rms_f, pot, field = run(dist, n, par)
     assert taken[0] <= accepted / TILES <= taken[1]
