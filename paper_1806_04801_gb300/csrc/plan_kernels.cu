@@ -15,21 +15,22 @@ namespace hsma {
 
 namespace {
 
-// Lifts a kernel's limit of dynamic shared memory to the most the device allows
-// beside its static part (an error where `bytes` is more).  The limit belongs to
-// the kernel: set to the call's own size, it made a larger launch of another
-// thread fail in between.
+// Lifts a kernel's limit of dynamic shared memory to the 227 KB that a block of
+// this part may have, less the kernel's static part (an error where `bytes` is
+// more).  The limit belongs to the kernel: set to the call's own size, it made a
+// larger launch of another thread fail in between.
 template <class K>
-cudaError_t allow_smem(K kernel, size_t bytes)
+cudaError_t allow_smem(K kernel, size_t bytes, size_t static_bytes = 0)
 {
-    int dev = 0, most = 0;
-    cudaFuncAttributes a;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (!e) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (!e) e = cudaFuncGetAttributes(&a, kernel);
-    if (e) return e;
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)std::max((size_t)most - a.sharedSizeBytes, bytes));
+                                (int)std::max<size_t>(227 * 1024 - static_bytes, bytes));
+}
+
+template <class K>
+size_t static_smem(K kernel)
+{
+    cudaFuncAttributes a{};
+    return cudaFuncGetAttributes(&a, kernel) == cudaSuccess ? a.sharedSizeBytes : 0;
 }
 
 constexpr double kPi = 3.14159265358979323846;
@@ -960,11 +961,11 @@ int build_pseudo_inverse(int K, int n, double *Wcol, double *Mp, double *cond_ho
         HSMA_LAUNCHED();
     }
     size_t smq = (size_t)K * sizeof(double);
-    HSMA_CUDA_TRY(allow_smem(qr_form_q_kernel, smq));
+    HSMA_CUDA_TRY(allow_smem(qr_form_q_kernel, smq, static_smem(qr_form_q_kernel)));
     qr_form_q_kernel<<<n, 256, smq, st>>>(Wcol, K, n, vtop, vv, Q1);
     HSMA_LAUNCHED();
     size_t smr = (size_t)n * sizeof(double);
-    HSMA_CUDA_TRY(allow_smem(r_inverse_kernel, smr));
+    HSMA_CUDA_TRY(allow_smem(r_inverse_kernel, smr, static_smem(r_inverse_kernel)));
     r_inverse_kernel<<<n, 128, smr, st>>>(Wcol, K, n, diag, Rinv);
     HSMA_LAUNCHED();
     long long tot = (long long)n * K;
