@@ -67,7 +67,14 @@ typedef struct hsma_plan_s *hsma_plan_t;
 typedef enum { HSMA_BC_PERIODIC = 0, HSMA_BC_GROUNDED = 1 } hsma_bc;
 
 /* Arithmetic of the update step.
- *  HSMA_FP64          everything in FP64 (parity form).
+ *  HSMA_FP64          FP64 accuracy throughout (parity form).  Near-field pairs
+ *                     are summed in fixed point: 62-bit coordinates, 63-bit
+ *                     charges in units of the largest of 256 sources, 1/r to
+ *                     2^-52, sums of 96 bits; close pairs, and sources whose
+ *                     charges differ so much that an FP64 loop would be more
+ *                     accurate, in FP64 proper.  The h^2 term of a thin dipole
+ *                     layer (1e-10 of it at the default Delta r) is computed
+ *                     in FP32, everything else in FP64.
  *  HSMA_FP32_ACC64    pair sums with FP32 differences (positions split into
  *                     two FP32 words), FP32 rsqrt and FP32 partial sums folded
  *                     into double-float accumulators; fit, mapping and energy
@@ -301,8 +308,10 @@ int hsma_shard_far(hsma_plan_t plan, const hsma_particles *x_q, const double *ph
  *   items_per_slot  work items per resident CTA slot (source chunks are sized
  *                   so that a call has about this many items per slot)
  *   ms              time measured by hsma_autotune (0 otherwise)
- * Defaults (no tuning entry for the call's work size): variant 14 for one
- * system, 17 for a batch, 48 items per slot (FP64: 24 items). */
+ * Defaults (no tuning entry for the call's work size): variant 13 for calls
+ * of less than 1e8 pairs, 17 for larger ones, 48 items per slot (FP64: 24
+ * items).  Small calls get fewer items than that: a chunk is at least one
+ * source tile. */
 typedef struct {
     int pair_variant;
     int items_per_slot;
@@ -427,8 +436,7 @@ void hsma_server_destroy(hsma_server_t srv);
  * Working memory -- about 32 (ns + nt) bytes and up to 160 MB of partial sums --
  * comes from the device's default memory pool.  Above 256 MiB it is given back
  * before the call returns; up to that the pool keeps it for a next call until
- * the process next synchronises (a stream, an event or the device).  Calls that
- * overlap each take their own.
+ * the process next synchronises (a stream, an event or the device).
  * Errors: HSMA_E_ARG, HSMA_E_OOM, HSMA_E_CUDA. */
 int hsma_coulomb_sum(int64_t ns, const double *src, int64_t nt, const double *tgt, double *pot,
                      double *field, int precision, void *stream);

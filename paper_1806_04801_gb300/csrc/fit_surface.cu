@@ -529,7 +529,10 @@ __global__ void __launch_bounds__(kSurf64Threads) surface_pairs_fp64_kernel(
 // a point dipole, and an h^2 term 1e-10 of it (dr = 1e-5 Rs) that FP32 holds
 // to the last FP64 bit.  The series leaves out (h/rho)^4 of the dipole, where
 // the literal difference of two 1/dr terms rounds at 2^-53 rho/h of it, so it
-// is the more accurate form while h <= 6.4e-4 rho (launch_surface_pairs).
+// is the more accurate form while h <= 6.4e-4 rho (launch_surface_pairs).  rho^2
+// and E below are rounded by up to 2^-53 (Rs/rho)^2, also less than that: at the
+// corners of boxes 1% to 30% inside their sphere, 540 to 2e5 directions, the
+// field's rms error is 0.001 to 0.94 times the literal form's.
 //
 // FP64 issue bounds both forms: 26 FP64 operations here per direction and
 // particle against 57 of the literal form.  A warp takes one particle and

@@ -530,14 +530,15 @@ __global__ void __launch_bounds__(kThreads, MINB) pair_fp32_kernel(PairArgs a)
 // its active cycles with one source per step; ALU 44%, issue slots 64%);
 // keeping the 64-bit additions apart from the multiplies was 7% slower, four
 // sources per step 6% faster than one.  Measured: near-sum phase of N = 9999
-// (1.96e9 pairs) 61.3 -> 10.5 ms, 3.2e10 -> 1.87e11 pairs/s; N = 1000 1.30 ->
-// 0.22 ms; grounded N = 3001 9.4 -> 1.56 ms.  Error against quad
+// (1.96e9 pairs) 61.3 -> 10.4 ms, 3.2e10 -> 1.89e11 pairs/s; N = 1000 1.30 ->
+// 0.21 ms; grounded N = 3001 9.4 -> 1.41 ms.  Error against quad
 // precision (N = 300..4000, both boundaries, three charge patterns): field
 // 1.8e-16..1.2e-15 of its norm against 4.7e-16..1.7e-15 before, potential
 // 1.4e-16..3.9e-15 against 3.5e-16..5.2e-15.  Those have charges of like size;
-// a tile with one far above the others goes native (fx_charges_fit; normal
-// charges now and then, and in a last tile of less than about 80: 527 -> 543 us
-// for 20011 sources x 3001 targets).
+// a tile with one far above the others goes native (fx_charges_fit), as fast as
+// the FP64 loop was (62 ms at N = 9999 with 1% of the charges 10^3 times the
+// rest); of tiles of normal charges that is one of less than about 80 now and
+// then (20011 sources x 3001 targets 529 -> 532..542 us).
 struct FxShared {
     double4_32a src[2][kTile64];       // staged sources (bulk copies land here)
     FxSource fx[kTile64];              // the tile being summed, in fixed point
