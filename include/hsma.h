@@ -434,9 +434,10 @@ void hsma_server_destroy(hsma_server_t srv);
  * field may be NULL.  precision as in hsma_precision (0 or 1).
  * stream: cudaStream_t or NULL.
  * Working memory -- about 32 (ns + nt) bytes and up to 160 MB of partial sums --
- * comes from the device's default memory pool.  Above 256 MiB it is given back
- * before the call returns; up to that the pool keeps it for a next call until
- * the process next synchronises (a stream, an event or the device).
+ * comes from a memory pool of the library.  The pool keeps up to 32 MiB per
+ * device until the process ends, and what a call of up to 256 MiB used until
+ * the process next synchronises (a stream, an event or the device); more than
+ * that is given back before the call returns.
  * Errors: HSMA_E_ARG, HSMA_E_OOM, HSMA_E_CUDA. */
 int hsma_coulomb_sum(int64_t ns, const double *src, int64_t nt, const double *tgt, double *pot,
                      double *field, int precision, void *stream);

@@ -1849,8 +1849,50 @@ int hsma_plan_load_tuning(hsma_plan_t pl, const char *cache_path)
 }
 
 // -------------------------------------------------------------- direct sums
-// Working memory that hsma_coulomb_sum may leave in the device's pool.
-constexpr size_t kCoulombKeep = (size_t)256 << 20;
+namespace {
+// Working memory of hsma_coulomb_sum.  A pool gives freed memory back at a wait
+// of any kind, and mapping it again takes 100-200 us, several times a small
+// call.  So the library has a pool of its own per device, which keeps up to
+// kCoulombKeep through any wait; what a call of up to kCoulombLate needs beyond
+// that it frees after its own wait, for a next call that comes before another
+// one, and more than that before it, so that it is gone when the call returns.
+// (1000 sources x 500 targets, a device-wide wait after each call: 250 us from
+// the default pool, 120 now; 117 without the waits.)
+constexpr size_t kCoulombKeep = (size_t)32 << 20;
+constexpr size_t kCoulombLate = (size_t)256 << 20;
+
+// That pool, or null where it cannot be had (the default one then serves).  A
+// reset of the device ends it with its context.  Called with g_scratch_mu held.
+cudaMemPool_t coulomb_pool(int dev)
+{
+    constexpr int kDevices = 64;
+    static struct {
+        cudaMemPool_t pool;
+        unsigned long long ctx;
+    } have[kDevices];
+    unsigned long long ctx = 0;
+    if (dev < 0 || dev >= kDevices || !current_context_id(&ctx)) return nullptr;
+    if (have[dev].pool && have[dev].ctx == ctx) return have[dev].pool;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    uint64_t keep = kCoulombKeep;
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) pool = nullptr;
+    if (pool && cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaMemPoolDestroy(pool);
+        pool = nullptr;
+    }
+    if (!pool) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    have[dev].pool = pool;
+    have[dev].ctx = ctx;
+    return pool;
+}
+}  // namespace
 
 int hsma_coulomb_sum(int64_t ns, const double *src, int64_t nt, const double *tgt, double *pot, double *field,
                      int precision, void *stream)
@@ -1888,21 +1930,16 @@ int hsma_coulomb_sum(int64_t ns, const double *src, int64_t nt, const double *tg
     };
     void *mem = nullptr;
     const size_t bytes = carve(nullptr);
-    // (cudaMalloc and the device-wide wait of cudaFree took 170 us a call)
-    HSMA_CUDA_TRY(dev_malloc_async(&mem, bytes, st));
+    HSMA_CUDA_TRY(dev_malloc_async(&mem, bytes, coulomb_pool(dev), st));
     carve(mem);
-    // Memory freed before a wait goes back to the device there.  Up to
-    // kCoulombKeep it is freed after this call's, so that the next call finds it
-    // in the pool unless the program has waited in between (1000 sources x 500
-    // targets 117 us, given back on every call 320; 20011 x 3001 527 and 707).
-    const bool keep = bytes <= kCoulombKeep;
+    const bool late = bytes <= kCoulombLate;
     int hst = 0;
     int rc = launch_coulomb(b, d, ns, src, nt, tgt, pot, field, precision, items, slots, st);
     if (!rc && cudaMemcpyAsync(&hst, b.status, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
         rc = HSMA_E_CUDA;
-    if (!keep) dev_free_async(mem, st);
+    if (!late) dev_free_async(mem, st);
     if (cudaStreamSynchronize(st) != cudaSuccess) rc = HSMA_E_CUDA;
-    if (keep) dev_free_async(mem, st);
+    if (late) dev_free_async(mem, st);
     if (!rc) rc = map_status(hst);
     if (rc == HSMA_OK && cudaGetLastError() != cudaSuccess) rc = HSMA_E_CUDA;
     return rc;

@@ -40,13 +40,14 @@ inline cudaError_t dev_free(void *p)
     g_alloc_calls.fetch_add(1, std::memory_order_relaxed);
     return cudaFree(p);
 }
-// Stream-ordered, from the device's default pool (which gives freed memory
-// back at the next synchronisation): for one call's working memory.
+// Stream-ordered, from `pool` (null: the device's default one): for one call's
+// working memory.
 template <class T>
-inline cudaError_t dev_malloc_async(T **p, size_t bytes, cudaStream_t st)
+inline cudaError_t dev_malloc_async(T **p, size_t bytes, cudaMemPool_t pool, cudaStream_t st)
 {
     g_alloc_calls.fetch_add(1, std::memory_order_relaxed);
-    return cudaMallocAsync(reinterpret_cast<void **>(p), bytes, st);
+    return pool ? cudaMallocFromPoolAsync(reinterpret_cast<void **>(p), bytes, pool, st)
+                : cudaMallocAsync(reinterpret_cast<void **>(p), bytes, st);
 }
 inline cudaError_t dev_free_async(void *p, cudaStream_t st)
 {
@@ -530,6 +531,7 @@ struct CoulombBuffers {
     double4_32a *s64, *t64;         // FP64 form
     float4 *partials;
 };
+bool current_context_id(unsigned long long *id);
 constexpr int kCoulombVariant = 13;  // FP32: two targets per thread, packed (pair.cu)
 SysDesc coulomb_shape(long long ns, long long nt, int precision, int slots);
 int launch_coulomb(const CoulombBuffers &b, const SysDesc &d, long long ns, const double *src, long long nt,

@@ -33,17 +33,6 @@
 
 namespace hsma {
 
-namespace {
-
-constexpr size_t kStaticScratchBytes = (size_t)HSMA_STATIC_SCRATCH_BYTES;
-static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
-
-constexpr int kMaxDevices = 64;
-std::mutex g_static_mu;
-void *g_scratch_addr[kMaxDevices] = {};
-unsigned long long g_scratch_ctx[kMaxDevices] = {};  // context id the address belongs to
-int g_num_sms[kMaxDevices] = {};
-
 // Process-unique id of the current context (cuCtxGetId), reached through the
 // runtime's driver entry-point table so that the library needs no link
 // against the driver library.  Returns false where the driver lacks it.
@@ -70,6 +59,17 @@ bool current_context_id(unsigned long long *id)
     if (!get_current || !get_id || get_current(&c) != CUDA_SUCCESS || !c) return false;
     return get_id(c, id) == CUDA_SUCCESS;
 }
+
+namespace {
+
+constexpr size_t kStaticScratchBytes = (size_t)HSMA_STATIC_SCRATCH_BYTES;
+static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
+
+constexpr int kMaxDevices = 64;
+std::mutex g_static_mu;
+void *g_scratch_addr[kMaxDevices] = {};
+unsigned long long g_scratch_ctx[kMaxDevices] = {};  // context id the address belongs to
+int g_num_sms[kMaxDevices] = {};
 
 size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 
