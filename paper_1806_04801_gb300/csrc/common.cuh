@@ -532,6 +532,7 @@ struct CoulombBuffers {
     float4 *partials;
 };
 bool current_context_id(unsigned long long *id);
+constexpr int kPackedFold = 64;      // sources per FP32 run of the packed loops, 32 in each lane
 constexpr int kCoulombVariant = 13;  // FP32: two targets per thread, packed (pair.cu)
 SysDesc coulomb_shape(long long ns, long long nt, int precision, int slots);
 int launch_coulomb(const CoulombBuffers &b, const SysDesc &d, long long ns, const double *src, long long nt,

@@ -117,6 +117,17 @@ __global__ void coulomb_init_kernel(SysDesc d, long long ns, SysDesc *dsys, long
     if (threadIdx.x >= 2 && threadIdx.x < 8) ctrl[threadIdx.x] = threadIdx.x < 5 ? INT_MAX : INT_MIN;
 }
 
+// Slot of source i of n for the packed FP32 loop, whose two lanes take the even
+// and the odd slots of a run of kPackedFold: the first half of a run's sources
+// in order to the one, the second half to the other.  In the caller's order the
+// lanes would take every other source, which sums charges of alternating sign
+// (a salt listed pair by pair) as two long sums of one sign each.
+__device__ __forceinline__ long long lane_run_slot(long long i, long long n)
+{
+    const int o = (int)(i % kPackedFold), m = (int)min((long long)kPackedFold, n - (i - o)), half = (m + 1) / 2;
+    return i - o + (o < half ? 2 * o : 2 * (o - half) + 1);
+}
+
 // Sources and targets into the pair kernels' records: FP32 word pairs, or FP64
 // records and the box of all coordinates (one pass over each; the first
 // `sblocks` blocks take the sources).
@@ -138,8 +149,9 @@ __global__ void __launch_bounds__(kSplitThreads) coulomb_split_kernel(long long 
         split_f64(x, hx, lx);
         split_f64(y, hy, ly);
         split_f64(z, hz, lz);
-        (is_src ? b.shi : b.thi)[i] = make_float4(hx, hy, hz, (float)q);
-        (is_src ? b.slo : b.tlo)[i] = make_float4(lx, ly, lz, 0.f);
+        const long long k = is_src ? lane_run_slot(i, ns) : i;
+        (is_src ? b.shi : b.thi)[k] = make_float4(hx, hy, hz, (float)q);
+        (is_src ? b.slo : b.tlo)[k] = make_float4(lx, ly, lz, 0.f);
         return;
     }
     if (live) (is_src ? b.s64 : b.t64)[i] = make_double4_32a(x, y, z, q);

@@ -45,7 +45,7 @@ constexpr int kTile64 = 256;
 constexpr int kFoldFx = 16;             // FxSums::gf fold interval (sources)
 constexpr int kStepFx = 4;              // sources per step
 constexpr int kFold = 32;               // potential fold interval (sources)
-constexpr int kFold2 = 64;              // packed loop: 32 sources per lane
+constexpr int kFold2 = kPackedFold;     // packed loop: 32 sources per lane
 constexpr bool kCpDouble = true;        // mode 1: two interleaved buffers, one barrier per tile
 constexpr float kFar = 1.0e4f;          // position of zero-charge padding sources
 
