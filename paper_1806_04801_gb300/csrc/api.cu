@@ -1923,7 +1923,7 @@ int hsma_coulomb_sum(int64_t ns, const double *src, int64_t nt, const double *tg
         b.t64 = cc.take<double4_32a>(n64 * nt);
         b.partials = cc.take<float4>(2 * (size_t)d.nchunks * nt);
         b.ns = cc.take<long long>(1);
-        b.ctrl = cc.take<int>(8);
+        b.ctrl = cc.take<int>(16);
         b.status = cc.take<int>(1);
         b.sys = cc.take<SysDesc>(1);
         return align_up(cc.off, 256);

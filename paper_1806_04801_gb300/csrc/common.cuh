@@ -468,8 +468,8 @@ struct PairArgs {
     int one_item = 0;               // 1: CTA b does work item b and exits (grid = total_items), so that
                                     // work on other streams gets SMs between items
     FxRange fx_part, fx_ext;  // FP64 form: formats for particle and for external targets
-    const int *fx_box = nullptr;  // FP64 form: if set, the formats come from this box of all coordinates
-                                  // (ordered FP32 keys, lows then highs: box_key)
+    const int *fx_box = nullptr;  // FP64 form: if set, the formats come from these boxes of the sources and of
+                                  // the targets (ordered FP32 keys, lows then highs of each: box_key)
     float4 *partials;       // 2 x float4 (FP32) or 1 x double4_32a (FP64) per record
     int *next_item;
     int *status;
@@ -525,7 +525,7 @@ int launch_finalize(const SysDesc *sys, int nsys, long long max_n, const int *pe
 struct CoulombBuffers {
     SysDesc *sys;
     long long *ns;
-    int *ctrl;    // [8] work counter, then the box keys
+    int *ctrl;    // [16] work counter, from [2] on the box keys
     int *status;
     float4 *shi, *slo, *thi, *tlo;  // FP32 form
     double4_32a *s64, *t64;         // FP64 form

@@ -97,7 +97,7 @@ StaticLayout layout_for(long long ns, long long nt, int nchunks, int precision)
     L.partials = put((size_t)nchunks * nt * 2 * sizeof(float4));
     put((size_t)nt * 4 * sizeof(double));  // not used: keeps the sizes that fit what they were
     L.ns = put(sizeof(long long));
-    L.ctrl = put(8 * sizeof(int));
+    L.ctrl = put(16 * sizeof(int));
     L.status = put(sizeof(int));
     L.sys = put(sizeof(SysDesc));
     L.end = o;
@@ -105,7 +105,7 @@ StaticLayout layout_for(long long ns, long long nt, int nchunks, int precision)
 }
 
 // Writes the work description, clears the counters and status and empties the
-// box of the coordinates.
+// boxes of the coordinates.
 __global__ void coulomb_init_kernel(SysDesc d, long long ns, SysDesc *dsys, long long *dns, int *ctrl, int *status)
 {
     if (threadIdx.x == 0) {
@@ -114,7 +114,7 @@ __global__ void coulomb_init_kernel(SysDesc d, long long ns, SysDesc *dsys, long
         *status = 0;
     }
     if (threadIdx.x < 2) ctrl[threadIdx.x] = 0;
-    if (threadIdx.x >= 2 && threadIdx.x < 8) ctrl[threadIdx.x] = threadIdx.x < 5 ? INT_MAX : INT_MIN;
+    if (threadIdx.x >= 2 && threadIdx.x < 14) ctrl[threadIdx.x] = (threadIdx.x - 2) % 6 < 3 ? INT_MAX : INT_MIN;
 }
 
 // Slot of source i of n for the packed FP32 loop, whose two lanes take the even
@@ -129,7 +129,7 @@ __device__ __forceinline__ long long lane_run_slot(long long i, long long n)
 }
 
 // Sources and targets into the pair kernels' records: FP32 word pairs, or FP64
-// records and the box of all coordinates (one pass over each; the first
+// records and the boxes of both (one pass over each; the first
 // `sblocks` blocks take the sources).
 constexpr int kSplitThreads = 256;
 __global__ void __launch_bounds__(kSplitThreads) coulomb_split_kernel(long long ns, const double *src, long long nt,
@@ -172,10 +172,11 @@ __global__ void __launch_bounds__(kSplitThreads) coulomb_split_kernel(long long 
         int m = red[threadIdx.x][0];
         for (int w = 1; w < kSplitThreads / 32; ++w)
             m = threadIdx.x < 3 ? min(m, red[threadIdx.x][w]) : max(m, red[threadIdx.x][w]);
+        int *key = &b.ctrl[(is_src ? 2 : 8) + threadIdx.x];
         if (threadIdx.x < 3)
-            atomicMin(&b.ctrl[2 + threadIdx.x], m);
+            atomicMin(key, m);
         else
-            atomicMax(&b.ctrl[2 + threadIdx.x], m);
+            atomicMax(key, m);
     }
 }
 

@@ -554,17 +554,23 @@ __device__ __forceinline__ unsigned abs_hi(double v) { return (unsigned)__double
 // 2^k, -1022 <= k <= 1023.
 __device__ __forceinline__ double exp2i(int k) { return __hiloint2double((k + 1023) << 20, 0); }
 
-// Formats for coordinates inside the box of the keys, from the box's centre;
-// native FP64 (scale 0) for a point, anything not finite, or a box so far
-// from the origin that its coordinates hold less than the formats.
+// Formats for coordinates inside the boxes of the keys (sources, targets), from
+// the centre of both; native FP64 (scale 0) for a point, anything not finite, or
+// boxes so far from the origin that the coordinates hold less than the formats.
 __device__ __forceinline__ FxRange range_of_box(const int *keys)
 {
     FxRange g;
-    float half = 0.f, mag = 0.f;
+    float half = 0.f, mag = 0.f, slo[3], shi[3], tlo[3], thi[3];
     double c[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const float lo = __int_as_float(box_key(keys[a])), hi = __int_as_float(box_key(keys[3 + a]));
+        const int ks = keys[a], kS = keys[3 + a], kt = keys[6 + a], kT = keys[9 + a];
+        slo[a] = __int_as_float(box_key(ks));
+        shi[a] = __int_as_float(box_key(kS));
+        tlo[a] = __int_as_float(box_key(kt));
+        thi[a] = __int_as_float(box_key(kT));
+        // by the keys, which order a NaN last
+        const float lo = __int_as_float(box_key(min(ks, kt))), hi = __int_as_float(box_key(max(kS, kT)));
         c[a] = 0.5 * ((double)lo + (double)hi);
         half = fmaxf(half, 0.5f * __fsub_ru(hi, lo));
         mag = fmaxf(mag, fmaxf(fabsf(lo), fabsf(hi)));
@@ -573,7 +579,8 @@ __device__ __forceinline__ FxRange range_of_box(const int *keys)
     if (!(half > 1e-30f && mag < half * 0x1p20f)) return g;
     // 2 half scale <= 2, with a bit in hand for the rounding of the origin
     const int e = (int)((unsigned)__float_as_int(half * 1.000001f) >> 23) - 126;  // half < 2^e
-    g.scale = exp2i(-e);
+    const int k = fx_halvings(slo, shi, tlo, thi, (float)kFxNearR * __int_as_float((e + 127) << 23));
+    g.scale = exp2i(-e - k);
     g.src_lim = 1073741823;
 #pragma unroll
     for (int a = 0; a < 3; ++a) g.origin[a] = rint(c[a] * g.scale * 0x1p30);

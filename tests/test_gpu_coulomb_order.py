@@ -5,10 +5,10 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-# Each FP32 partial sum rounds at its own size.  Charges of alternating sign keep those sums at a few terms, random signs
-# at the square root of their number; so the alternating order's error is no larger than a random order's (half again for
-# the scatter of 300 targets).  The targets are away from the sources: beside them a few closest pairs, the same in every
-# order, make up most of the field's error.
+# Each FP32 partial sum rounds at its own size.  Charges of alternating sign keep those sums at a few terms, random
+# signs at the square root of their number; so the alternating order's error is no larger than a random order's (half
+# again for the scatter of 300 targets).  The targets are away from the sources: beside them a few closest pairs, the
+# same in every order, make up most of the field's error.
 @pytest.mark.parametrize("away", [2.0, 20.0])
 @pytest.mark.parametrize("n", [64, 250, 2000, 20001])
 def test_alternating_charges_are_summed_as_well_as_random_ones(n, away):
