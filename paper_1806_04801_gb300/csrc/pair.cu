@@ -538,7 +538,7 @@ __global__ void __launch_bounds__(kThreads, MINB) pair_fp32_kernel(PairArgs a)
 // a tile with one far above the others goes native (fx_charges_fit), as fast as
 // the FP64 loop was (62 ms at N = 9999 with 1% of the charges 10^3 times the
 // rest); of tiles of normal charges that is one of less than about 80 now and
-// then (20011 sources x 3001 targets 529 -> 532..542 us).
+// then (20011 sources x 3001 targets 529 -> 531 us).
 struct FxShared {
     double4_32a src[2][kTile64];       // staged sources (bulk copies land here)
     FxSource fx[kTile64];              // the tile being summed, in fixed point
